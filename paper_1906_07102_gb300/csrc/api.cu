@@ -86,7 +86,7 @@ namespace lmg {
 void free_plan(lmg_plan* p) {
   if (!p) return;
   void* ptrs[] = {p->d_table, p->d_h, p->hist, p->offsets, p->rank, p->partial, p->recs,
-                  p->items, p->counters, p->spill, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
+                  p->items, p->cuts, p->counters, p->spill, p->parts, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->fft_ok) cufftDestroy(p->fft);
@@ -115,6 +115,10 @@ SweepArgs sweep_args(const lmg_plan* p) {
   a.W = p->W;
   a.dtype = p->dtype;
   a.item_cap = p->item_cap;
+  a.direct = p->direct ? 1 : 0;
+  a.part_cap = p->part_cap;
+  a.cuts = p->cuts;
+  a.parts = p->parts;
   a.nvis = p->nvis;
   a.frac = p->frac;
   return a;
@@ -306,8 +310,11 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   p->n_strips = int(N / strip);
   const size_t rs = dtype == LMG_C128 ? 8 : 4;
   p->Wp = table_stride(p->W, dtype);
-  const int nblk = int((N + opt.min_rows_per_block - 1) / opt.min_rows_per_block);
-  p->item_cap = p->n_strips * nblk + int((2 * max_vis) / opt.min_item_target) + 2;
+  p->direct = opt.direct && grid_direct(N, dtype);
+  p->auto_target = opt.min_item_target == 0;
+  p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block,
+                               p->auto_target ? item_target_for(max_vis) : opt.min_item_target));
+  p->part_cap = dtype == LMG_C64 && p->auto_target ? part_bound(max_vis) : 0;
   if (inject_fault("item_cap")) p->item_cap = 1;
   const long long L = (long long)p->n_strips * N;
   p->nchunks = bin_scan_chunks(L);
@@ -355,7 +362,11 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
       (rc = dalloc(&p->offsets, size_t(L) + 1, "offsets")) || (rc = dalloc(&p->rank, size_t(max_vis), "ranks")) ||
       (rc = dalloc(&p->partial, size_t(p->nchunks), "scan")) || (rc = dalloc(&p->recs, size_t(2 * max_vis), "records")) ||
       (rc = dalloc(&p->items, size_t(p->item_cap), "items")) || (rc = dalloc(&p->counters, kNumCounters, "counters")) ||
-      (rc = dalloc(reinterpret_cast<unsigned char**>(&p->spill), size_t(p->item_cap) * ring_slots(p->W) * strip * c2, "spill")) ||
+      (!p->direct &&
+       (rc = dalloc(reinterpret_cast<unsigned char**>(&p->spill), size_t(p->item_cap) * ring_slots(p->W) * strip * c2, "spill"))) ||
+      (p->part_cap > 0 &&
+       ((rc = dalloc(&p->cuts, size_t(p->part_cap), "cut pairs")) ||
+        (rc = dalloc(&p->parts, size_t(p->part_cap) * size_t(p->W + 1) * 2 * size_t(strip), "sums of parts")))) ||
       (dtype == LMG_C128 && (rc = dalloc(&p->frac, size_t(max_vis), "quantisation residuals"))) ||
       (opt.work_grid && (rc = dalloc(reinterpret_cast<unsigned char**>(&p->work), size_t(N) * size_t(N) * c2, "work grid"))) ||
       (opt.work_grid && !p->xform &&
@@ -402,15 +413,15 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   p->smem_grid = sweep_smem_bytes(p->W, dtype, p->Ms, p->tab_smem_grid, false, p->warps_grid);
   p->smem_degrid = sweep_smem_bytes(p->W, dtype, p->Ms, p->tab_smem_degrid, true, p->warps_degrid);
   for (int accum = 0; accum <= (dtype == LMG_C64 ? 1 : 0); ++accum) {
-    if (sweep_set_smem_limits(p->W, dtype, accum, p->smem_grid, false, p->interp >= 2) ||
-        sweep_occupancy(p->W, dtype, accum, p->smem_grid, false, p->interp >= 2, p->warps_grid, &bps)) {
+    if (sweep_set_smem_limits(p->W, dtype, accum, p->smem_grid, false, p->interp >= 2, p->direct) ||
+        sweep_occupancy(p->W, dtype, accum, p->smem_grid, false, p->interp >= 2, p->direct, p->warps_grid, &bps)) {
       free_plan(p);
       return cuda_error(cudaGetLastError(), "sweep kernel attributes");
     }
     (accum ? p->blocks_grid_comp : p->blocks_grid) = p->sms * (bps > 0 ? bps : 1);
   }
-  if (sweep_set_smem_limits(p->W, dtype, 0, p->smem_degrid, true, p->interp >= 2) ||
-      sweep_occupancy(p->W, dtype, 0, p->smem_degrid, true, p->interp >= 2, p->warps_degrid, &bps)) {
+  if (sweep_set_smem_limits(p->W, dtype, 0, p->smem_degrid, true, p->interp >= 2, false) ||
+      sweep_occupancy(p->W, dtype, 0, p->smem_degrid, true, p->interp >= 2, false, p->warps_degrid, &bps)) {
     free_plan(p);
     return cuda_error(cudaGetLastError(), "sweep kernel attributes");
   }
@@ -463,8 +474,12 @@ int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64
   a.n_strips = p->n_strips;
   a.strip = p->strip;
   a.rows_per_block = p->rows_per_block;
-  a.item_target = p->item_target;
+  a.item_target = p->auto_target ? item_target_within(nvis, p->n_strips, int(p->N), p->rows_per_block, p->item_cap)
+                                 : p->item_target;
   a.item_cap = p->item_cap;
+  a.skip_empty = p->direct ? 1 : 0;
+  a.cuts = p->cuts;
+  a.part_cap = p->part_cap;
   a.max_blocks = p->sms * 8;
   a.hist = p->hist;
   a.offsets = p->offsets;

@@ -601,6 +601,7 @@ int lmg_batch_create(int n_chan, const lmg_table* const* tables, const int64_t* 
   PlanOptions opt;
   opt.min_rows_per_block = 64;
   opt.min_item_target = 256;
+  opt.direct = false;
   opt.work_grid = false;
   opt.fft = false;
   for (int c = 0; c < n_chan; ++c) {

@@ -13,7 +13,7 @@
 //                    the sweeps stage together -- to the pair's range, dealt so that any 32
 //                    consecutive records sample the whole pair (see dealt_position).
 //   4. k_make_items  per strip and block of rows: items holding about item_target records,
-//                    cut at even rows so that the sweeps' row groups are these pairs.
+//                    of whole row pairs (the sweeps' row groups) or parts of a dense pair.
 // With a track layout (positions stored sample-major, k = t * tracks + b) passes 1 and 3
 // follow each track instead (k_bin_count_tracks, k_bin_scatter_tracks).
 #include <cuda_runtime.h>
@@ -395,46 +395,133 @@ __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale
   }
 }
 
-// One CTA per (strip, block of rows): the block's row offsets are staged in shared memory
-// and the block is cut into items of about `target` records each (at least one item per
-// block) by binary searches there, one item per thread. Items with more than target/2
-// records are placed from the front of the array and the others from the back, so that
-// the sweeps (which take items front to back, then back to front) start the heavy ones
-// first.
+// One CTA per (strip, block of rows). Thread i holds row pair i of the block. Pairs are joined
+// with their neighbours into items of equal counts, about target records each. With a
+// target below kDenseUnit (few visibilities) they are joined in units of the pairs that W - 1
+// rows take, up to kDenseUnit records: items of whole units meet in a cell at most two at a time,
+// so that their sums do not depend on which is added first. Elsewhere items are cut at any pair,
+// and a pair with 8 target records or more is cut into parts of 4 to 8 target records, one item
+// each: a warp sweeps an item alone, and one dense pair near the uv origin, 40 times the target,
+// is otherwise a serial chain that the whole launch waits for (4.1M visibilities on a 256^2 grid:
+// 512 such items kept a fifth of the resident warps busy, and degridding took 4.4 ms, 0.43 with
+// the cut).
+// Items per block are at most 1 + count / target: a cut pair of n >= 8 target records gives at
+// most n / (4 target) parts and one more boundary between joined pairs.
+// Items with more than target/2 records are placed from the front of the array and the others
+// from the back, so that the sweeps (which take items front to back, then back to front)
+// start the heavy ones first. skip_empty: items without records are left out (the gridding
+// sweep then adds into a zeroed grid; otherwise they store their rows' zeros).
 constexpr int kMaxRowsPerBlock = 512;
+constexpr int kItemThreads = kMaxRowsPerBlock / 2;
+constexpr int kDenseUnit = 512;
+// Parts that plain float32 gridding sums in one chain. Its accuracy on dense cells follows the
+// length of its chains; 4.1M visibilities on a 256^2 grid, W = 12, relative image error and time:
+// uncut 4.9e-6 in 4.40 ms, 12 parts 1.8e-6 in 1.86, 8 parts 1.2e-6 in 1.23, 4 parts 6.3e-7 in
+// 0.74, one 4.4e-7 in 0.40; compensated 2.5e-7 in 1.17 (9.9 uncut). Eight keep the plain sums as
+// clearly apart from the compensated ones as tests/test_gpu_precision.py holds them (3 times).
+constexpr int kChain = 8;
 
-__global__ void k_make_items(const int* __restrict__ offsets, int N, int n_strips, int rows_per_block,
-                             int target, Item* __restrict__ items, int* __restrict__ counters, int cap) {
-  __shared__ int s_off[kMaxRowsPerBlock + 1];
+__device__ __forceinline__ void put_item(const Item& it, int target, Item* __restrict__ items,
+                                         int* __restrict__ counters, int cap) {
+  int slot;
+  if (2 * it.nrec > target) slot = atomicAdd(counters + kCntItems, 1);
+  else slot = cap - 1 - atomicAdd(counters + kCntItemsBack, 1);
+  if (slot >= 0 && slot < cap) items[slot] = it;
+  else atomicOr(counters + kCntStatus, kStatusItemOverflow);
+}
+
+__global__ void __launch_bounds__(kItemThreads)
+    k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty,
+                 Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
+  __shared__ int s_part0;
+  __shared__ int s_off[kItemThreads + 1];  // offset of each pair's first record
+  __shared__ int s_pre[kItemThreads];      // records of joined pairs before each pair
+  __shared__ unsigned s_start[kItemThreads / 32 + 1], s_cut[kItemThreads / 32];
+  __shared__ int s_warp[kItemThreads / 32];
   const int nblk = (N + rows_per_block - 1) / rows_per_block;
   const int s = blockIdx.x / nblk, b = blockIdx.x % nblk;
-  const int rb = b * rows_per_block, re = min(N, rb + rows_per_block);
-  const int* off = offsets + static_cast<long long>(s) * N;
-  for (int r = threadIdx.x; r <= re - rb; r += blockDim.x) s_off[r] = off[rb + r];
+  const int rb = b * rows_per_block, np = (min(N, rb + rows_per_block) - rb) / 2;
+  const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = blockDim.x >> 5;
+  const int* off = offsets + static_cast<long long>(s) * N + rb;
+  for (int k = i; k <= np; k += blockDim.x) s_off[k] = off[2 * k];
   __syncthreads();
-  const int o0 = s_off[0], count = s_off[re - rb] - o0;
-  const int m = max(1, (count + target - 1) / target);
-  // first row (relative) whose offset reaches the k-th cut
-  auto cut = [&](int k) {
-    if (k <= 0) return 0;
-    if (k >= m) return re - rb;
-    const long long goal = o0 + (static_cast<long long>(count) * k) / m;
-    int lo = 0, hi = re - rb;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (s_off[mid] >= goal) hi = mid;
-      else lo = mid + 1;
-    }
-    return lo & ~1;  // even rows: the sweeps' row groups are the binned row pairs
+  // unit of pair i: u pairs, the last unit of the block with the remainder
+  const int u = target < kDenseUnit ? max(1, W >> 1) : 1, nu = max(1, np / u);
+  auto unit_first = [&](int k) { return min(k / u, nu - 1) * u; };
+  auto dense_unit = [&](int first) {
+    const int end = first / u == nu - 1 ? np : first + u;
+    return u == 1 || s_off[end] - s_off[first] > kDenseUnit;
   };
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
-    const int r0 = cut(k), r1 = cut(k + 1);
-    const int n = s_off[r1] - s_off[r0];
-    int slot;
-    if (2 * n > target) slot = atomicAdd(counters + kCntItems, 1);
-    else slot = cap - 1 - atomicAdd(counters + kCntItemsBack, 1);
-    if (slot >= 0 && slot < cap) items[slot] = Item{s, rb + r0, rb + r1, n};
-    else atomicOr(counters + kCntStatus, kStatusItemOverflow);
+  const bool in = i < np;
+  const int first = in ? unit_first(i) : 0;
+  const bool dense = in && dense_unit(first);
+  const int n = in ? s_off[i + 1] - s_off[i] : 0;
+  const bool cut = dense && n >= 8 * target;
+  const int nj = cut ? 0 : n;
+  int x = nj;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[warp] = x;
+  const unsigned cm = __ballot_sync(0xffffffffu, cut);
+  if (lane == 0) s_cut[warp] = cm;
+  __syncthreads();
+  int base = 0, joined = 0;
+  for (int k = 0; k < nw; ++k) {
+    base += k < warp ? s_warp[k] : 0;
+    joined += s_warp[k];
+  }
+  const int pre = base + x - nj;
+  // joined pairs go to m items of equal counts, as far as the places to cut allow
+  const int m_items = max(1, (joined + target - 1) / target);
+  auto item_of = [&](int r) { return joined ? static_cast<int>(static_cast<long long>(r) * m_items / joined) : 0; };
+  s_pre[i] = pre;
+  __syncthreads();
+  // a joined item starts at the block's first pair, after a cut pair, and where the running
+  // count passes into the next item's share
+  bool start = in && (cut || i == 0);
+  if (in && !start && (dense || i == first)) {
+    const int f = unit_first(i - 1), p = dense_unit(f) ? i - 1 : f;
+    start = ((s_cut[(i - 1) >> 5] >> ((i - 1) & 31)) & 1u) || item_of(pre) != item_of(s_pre[p]);
+  }
+  const unsigned sm = __ballot_sync(0xffffffffu, start);
+  if (lane == 0) s_start[warp] = sm;
+  __syncthreads();
+  if (start && !cut) {
+    int w = warp;
+    unsigned m = lane == 31 ? 0u : s_start[w] & (0xffffffffu << (lane + 1));
+    while (!m && ++w < nw) m = s_start[w];
+    const int end = m ? 32 * w + __ffs(m) - 1 : np;
+    const int cnt = s_off[end] - s_off[i];
+    if (cnt > 0 || !skip_empty)
+      put_item(Item{s, rb + 2 * i, rb + 2 * end, cnt, s_off[i], 2 * (end - i), -1, cnt}, target, items, counters, cap);
+  }
+  // cut pairs, one after another, their parts over the threads
+  for (int w = 0; w < nw; ++w) {
+    for (unsigned m = s_cut[w]; m; m &= m - 1) {
+      const int p = 32 * w + __ffs(m) - 1;
+      const int o0 = s_off[p], cnt = s_off[p + 1] - o0, parts = cnt / (4 * target);
+      int part0 = -1;
+      if (cuts != nullptr) {
+        if (i == 0) {
+          const int q = atomicAdd(counters + kCntParts, parts);
+          s_part0 = q + parts <= part_cap ? q : -1;
+          if (s_part0 >= 0) cuts[atomicAdd(counters + kCntCuts, 1)] = Cut{s, rb + 2 * p, q, parts};
+          else atomicOr(counters + kCntStatus, kStatusItemOverflow);
+        }
+        __syncthreads();
+        part0 = s_part0;
+        __syncthreads();
+      }
+      for (int k = i; k < parts; k += blockDim.x) {
+        const int a = o0 + static_cast<int>(static_cast<long long>(cnt) * k / parts);
+        const int e = o0 + static_cast<int>(static_cast<long long>(cnt) * (k + 1) / parts);
+        const int ce = o0 + static_cast<int>(static_cast<long long>(cnt) * min(k + kChain, parts) / parts);
+        const int chain = k % kChain == 0 ? ce - a : 0;
+        put_item(Item{s, rb + 2 * p, rb + 2 * p + 2, e - a, a, k == 0 ? 2 : 0, part0 < 0 ? -1 : part0 + k, chain}, target, items, counters, cap);
+      }
+    }
   }
 }
 
@@ -472,9 +559,40 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const int nblk = (a.N + a.rows_per_block - 1) / a.rows_per_block;
   const int ntask = a.n_strips * nblk;
   if (a.rows_per_block > kMaxRowsPerBlock) return -1;
-  k_make_items<<<ntask, 128, 0, st>>>(a.offsets, a.N, a.n_strips, a.rows_per_block, a.item_target,
-                                                   a.items, a.counters, a.item_cap);
+  const int item_threads = a.rows_per_block <= 256 ? 128 : kItemThreads;
+  k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty, a.items,
+                                               a.counters, a.item_cap, a.cuts, a.part_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// Records per work item. A warp sweeps an item alone, so a call with few visibilities wants
+// small items: with 512 records each, the 20,000 visibilities of a 256^2 grid made 40 items for
+// 2432 resident warps and the sweep took 50 us, as long as one item does. 32 warps per SM give
+// each warp about two items; from 32 records down an item is all start-up (its grid rows and
+// offsets); above 512 nothing is gained (best of {256 .. 2048} on 4.1M-visibility tracks).
+int item_target_for(long long nvis) {
+  const long long t = nvis / (32 * kSms);
+  return static_cast<int>(t < 32 ? 32 : (t > 512 ? 512 : t));
+}
+
+// Work items that nvis positions (two records each at most) can make (see k_make_items).
+long long item_bound(long long nvis, int n_strips, int N, int rows_per_block, int target) {
+  const long long nblk = (N + rows_per_block - 1) / rows_per_block;
+  return n_strips * nblk + 2 * nvis / target + 2;
+}
+
+// A cut pair's n records give at most n / (4 target) parts, and nvis positions two records
+// each; nvis / item_target_for(nvis) is largest at max_vis or where the target passes 33.
+int part_bound(long long max_vis) {
+  const long long n = max_vis / 32 <= 32 * kSms ? max_vis / 32 : 33 * kSms;
+  return static_cast<int>((n > max_vis / 512 ? n : max_vis / 512) / 2 + 1);
+}
+
+int item_target_within(long long nvis, int n_strips, int N, int rows_per_block, int cap) {
+  const long long room = cap - item_bound(0, n_strips, N, rows_per_block, 1);
+  const long long least = room > 0 ? (2 * nvis + room - 1) / room : 0;
+  const int t = item_target_for(nvis);
+  return least > t ? static_cast<int>(least) : t;
 }
 
 int bin_scan_chunks(long long L) { return static_cast<int>((L + kScanChunk - 1) / kScanChunk); }

@@ -28,9 +28,20 @@ __host__ __device__ __forceinline__ int rec_pack(int row, int xrel) { return (ro
 __host__ __device__ __forceinline__ int rec_xrel(int rx) { return static_cast<int>(static_cast<signed char>(rx & 0xff)); }
 __host__ __device__ __forceinline__ int rec_row(int rx) { return static_cast<int>(static_cast<unsigned>(rx) >> 8); }
 
-// Work item: rows [r0, r1) of one strip holding nrec records.
-struct Item {
+// Work item: the records [rb, rb + nrec) of rows [r0, r1) of one strip. A pair of rows with
+// many records is cut into several items over the same rows (parts); own (the rows whose final
+// sums the item stores itself, r1 - r0 or 0) is non-zero for the first of them only. part is
+// the part's place in the buffer that compensated sums of parts are kept in, -1 otherwise.
+// Plain float32 gridding takes kChain parts of a pair as one chain: chain is the chain's records
+// for its first part, 0 for the others (which it skips), and nrec for the other items.
+struct alignas(16) Item {
   int strip, r0, r1, nrec;
+  int rb, own, part, chain;
+};
+
+// A cut pair of rows r0, r0 + 1: its parts' places are [part0, part0 + parts).
+struct alignas(16) Cut {
+  int strip, r0, part0, parts;
 };
 
 template <typename R> struct Cplx;

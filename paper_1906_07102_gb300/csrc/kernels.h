@@ -22,6 +22,9 @@ __host__ __device__ constexpr int table_stride(int W, int dtype) {
 
 struct Rec;
 struct Item;
+struct Cut;
+
+constexpr int kSms = 152;  // GB300
 
 // counters[] slots (device ints, reset by bin_launch)
 enum {
@@ -31,6 +34,8 @@ enum {
   kCntItemsBack = 3,   // items placed from the back (light)
   kCntGridWork = 4,    // work counter of the gridding sweep
   kCntDegridWork = 5,  // work counter of the degridding sweep
+  kCntCuts = 6,        // cut row pairs
+  kCntParts = 7,       // their parts
   kNumCounters = 8
 };
 
@@ -45,6 +50,7 @@ struct BinArgs {
   double scale2;  // N * pixel_scale * 2^32
   int W, N, n_strips, strip;  // strip: columns per strip (strip_width)
   int rows_per_block, item_target, item_cap;
+  int skip_empty;  // leave out work items without records (gridding into a zeroed grid)
   int max_blocks;
   int* hist;       // n_strips * N
   int* offsets;    // n_strips * N + 1
@@ -52,6 +58,8 @@ struct BinArgs {
   int* partial;    // scan chunk sums
   Rec* recs;       // 2 * max_vis
   Item* items;     // item_cap
+  Cut* cuts;       // part_cap or NULL (no compensated gridding): the cut row pairs
+  int part_cap;
   int* counters;   // 8
   double2* frac;   // max_vis or NULL: per visibility (u_q - u, v_q - v) in cells, the residual
                    // of the 2^-32 quantisation (float64 plans: exact table fractions)
@@ -72,6 +80,16 @@ int xform_model_launch(const void* image, void* grid, void* scratch, const float
 
 int bin_launch(const BinArgs& a, cudaStream_t st);
 int bin_scan_chunks(long long L);
+int item_target_for(long long nvis);
+long long item_bound(long long nvis, int n_strips, int N, int rows_per_block, int target);
+// Parts of cut row pairs that up to max_vis positions can make.
+int part_bound(long long max_vis);
+// item_target_for, raised until item_bound stays within cap items.
+int item_target_within(long long nvis, int n_strips, int N, int rows_per_block, int cap);
+// Gridding by adding into a zeroed grid instead of storing whole rows and adding spill rows:
+// where the grid stays in L2 (129 MB, half of it at most), zeroing and vector reductions cost
+// no DRAM traffic, and small items need no spill buffer and no pass over it.
+constexpr bool grid_direct(long long N, int dtype) { return N * N * (dtype ? 16 : 8) <= (48ll << 20); }
 
 struct SweepArgs {
   const Rec* recs;
@@ -85,6 +103,7 @@ struct SweepArgs {
   int dtype;          // 0 float, 1 double
   int accum;          // 0 plain, 1 compensated (float only)
   int item_cap;
+  int direct;         // gridding adds into a zeroed grid (grid_direct); else rows are stored once
   int grid_blocks;    // persistent CTAs
   int warps;          // warps per CTA (1..8)
   int table_in_smem;
@@ -92,7 +111,10 @@ struct SweepArgs {
   const void* vis;
   const void* weights;
   void* grid;
-  void* spill;        // item_cap * ring rows * strip complex
+  void* spill;        // item_cap * ring rows * strip complex (not used when direct)
+  int part_cap;
+  const Cut* cuts;    // compensated gridding: cut row pairs and the sums of their parts,
+  float2* parts;      // [part][W + 1 rows][sum, rounding error][strip]
   // degridding
   const void* grid_in;
   void* vis_out;
@@ -108,11 +130,11 @@ int degrid_launch(const SweepArgs& a, cudaStream_t st, bool zero_out = true);
 // Shared memory a sweep CTA needs (bytes) and CTAs per SM that fit; used to size launches.
 size_t sweep_smem_bytes(int W, int dtype, int Ms, bool table_in_smem, bool degrid, int warps);
 // ext: the kernels of the extended lookups (interp >= 2: Lagrange, direct calculation).
-int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext);
-int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, int warps,
+int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct);
+int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct, int warps,
                     int* blocks_per_sm);
 // Kernel of the extended lookups (sweep_ext.cu).
-void* sweep_kernel_ext(int W, int dtype, int accum, bool degrid);
+void* sweep_kernel_ext(int W, int dtype, int accum, bool degrid, bool direct);
 // Warps per CTA and table placement so that a CTA's shared memory stays within `limit`.
 int sweep_config(int W, int dtype, int Ms, bool degrid, size_t limit, bool* table_in_smem, int* warps);
 

@@ -60,8 +60,11 @@ struct lmg_plan {
   int W = 0, Ms = 0, interp = 1, dtype = 0, Wp = 0;
   int64_t n_image = 0, N = 0;
   double x0 = 0, pixel_scale = 0, scale2 = 0;
-  // work items: blocks of 64 rows of a strip cut into items of ~512 records (measured best of
-  // {64..512} x {256..2048} on the 4.1M-visibility tracks: better balance of the persistent sweeps)
+  // work items: blocks of 64 rows of a strip cut into items of item_target records, or of
+  // item_target_for(nvis) (up to 512: best of {64..512} rows x {256..2048} records on the
+  // 4.1M-visibility tracks) when auto_target
+  bool auto_target = true;
+  bool direct = false;  // gridding adds into a zeroed grid (grid_direct); no spill buffer
   int n_strips = 0, strip = 64, rows_per_block = 64, item_target = 512, item_cap = 0, nchunks = 0;
   int64_t max_vis = 0, nvis = -1;
   int device = 0, sms = 0;
@@ -78,6 +81,10 @@ struct lmg_plan {
   int* partial = nullptr;
   lmg::Rec* recs = nullptr;
   lmg::Item* items = nullptr;
+  // compensated gridding: cut row pairs and the sums of their parts
+  int part_cap = 0;
+  lmg::Cut* cuts = nullptr;
+  float2* parts = nullptr;
   int* counters = nullptr;
   void* spill = nullptr;
   double2* frac = nullptr;   // float64 plans: quantisation residual of every position
@@ -102,7 +109,8 @@ namespace lmg {
 // smallest bin parameters the tuner may choose, and no per-plan work grid or FFT plan.
 struct PlanOptions {
   int min_rows_per_block = 64;
-  int min_item_target = 512;
+  int min_item_target = 0;  // 0: sized by the visibility count
+  bool direct = true;       // allow gridding by adding into a zeroed grid
   bool work_grid = true;
   bool fft = true;
 };

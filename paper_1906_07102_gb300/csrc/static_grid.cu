@@ -24,15 +24,15 @@ namespace {
 constexpr int64_t kMaxVis = LMG_STATIC_MAX_VIS;
 constexpr int kMaxN = LMG_STATIC_MAX_N;
 constexpr int kMaxOversample = LMG_STATIC_MAX_OVERSAMPLE;
-constexpr int kRowsPerBlock = 256;
-constexpr int kItemTarget = 1024;
+constexpr int kRowsPerBlock = 64;
+constexpr int kMinItemTarget = 32;
 constexpr int kStaticStrip = strip_width(LMG_C64);  // complex64 only
 constexpr int kMaxStrips = kMaxN / kStaticStrip;
 constexpr long long kMaxBuckets = static_cast<long long>(kMaxStrips) * kMaxN;
 constexpr int kMaxItems = kMaxStrips * ((kMaxN + kRowsPerBlock - 1) / kRowsPerBlock) +
-                          static_cast<int>((2 * kMaxVis) / kItemTarget) + 2;
+                          static_cast<int>(2 * kMaxVis / kMinItemTarget) + 2;  // item_bound
 constexpr int kMaxWp = table_stride(16, LMG_C64);  // float row stride for W <= 16
-constexpr int kMaxRing = 18;    // ring slots for W = 16
+static_assert(grid_direct(kMaxN, LMG_C64), "every size adds into a zeroed grid: no spill buffer");
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
 
@@ -45,8 +45,7 @@ constexpr size_t kOffPartial = kOffOffsets + up256(sizeof(int) * (kMaxBuckets + 
 constexpr size_t kOffRecs = kOffPartial + up256(sizeof(int) * (kMaxBuckets / 4096 + 2));
 constexpr size_t kOffItems = kOffRecs + up256(sizeof(Rec) * 2 * kMaxVis);
 constexpr size_t kOffCounters = kOffItems + up256(sizeof(Item) * kMaxItems);
-constexpr size_t kOffSpill = kOffCounters + up256(sizeof(int) * kNumCounters);
-constexpr size_t kScratchBytes = kOffSpill + up256(sizeof(float2) * kMaxItems * kMaxRing * kStaticStrip);
+constexpr size_t kScratchBytes = kOffCounters + up256(sizeof(int) * kNumCounters);
 
 // The working memory: allocated when the library is loaded, on every device that loads
 // it, and held until the process exits.
@@ -170,8 +169,7 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   }
 
   const int n_strips = int(N / kStaticStrip);
-  const int nblk = int((N + kRowsPerBlock - 1) / kRowsPerBlock);
-  const int item_cap = n_strips * nblk + int((2 * nvis) / kItemTarget) + 2;
+  const int item_cap = kMaxItems;
   BinArgs b{};
   b.uv = uv;
   b.nvis = nvis;
@@ -181,8 +179,9 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   b.n_strips = n_strips;
   b.strip = kStaticStrip;
   b.rows_per_block = kRowsPerBlock;
-  b.item_target = kItemTarget;
+  b.item_target = item_target_within(nvis, n_strips, int(N), kRowsPerBlock, item_cap);
   b.item_cap = item_cap;
+  b.skip_empty = 1;
   b.max_blocks = s->sms * 8;
   b.rank = reinterpret_cast<int2*>(base + kOffRank);
   b.hist = reinterpret_cast<int*>(base + kOffHist);
@@ -199,8 +198,8 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
     return set_error(LMG_EUNSUPPORTED, "sweep shared memory does not fit for this W");
   const size_t smem = sweep_smem_bytes(W, LMG_C64, Ms, tab_smem, false, warps);
   const bool ext = t->interp >= 2;
-  if (sweep_set_smem_limits(W, LMG_C64, 0, smem, false, ext) ||
-      sweep_occupancy(W, LMG_C64, 0, smem, false, ext, warps, &bps))
+  if (sweep_set_smem_limits(W, LMG_C64, 0, smem, false, ext, true) ||
+      sweep_occupancy(W, LMG_C64, 0, smem, false, ext, true, warps, &bps))
     return set_error(LMG_ECUDA, std::string("sweep kernel attributes: ") + cudaGetErrorString(cudaGetLastError()));
   SweepArgs a{};
   a.recs = b.recs;
@@ -218,13 +217,13 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   a.dtype = LMG_C64;
   a.accum = 0;
   a.item_cap = item_cap;
+  a.direct = 1;
   a.grid_blocks = s->sms * (bps > 0 ? bps : 1);
   a.warps = warps;
   a.table_in_smem = tab_smem ? 1 : 0;
   a.vis = vis;
   a.weights = weights;
   a.grid = grid;
-  a.spill = base + kOffSpill;
   a.nvis = nvis;
   if (grid_launch(a, st) != 0) return set_error(LMG_ECUDA, std::string("gridding launch: ") + cudaGetErrorString(cudaGetLastError()));
   return LMG_OK;

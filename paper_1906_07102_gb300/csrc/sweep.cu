@@ -1,5 +1,7 @@
 // Single-plan gridding and degridding: the nearest / linear table kernels (the extended
 // lookups are compiled in sweep_ext.cu), the spill pass, launch configuration.
+#include <algorithm>
+
 #include "sweep_body.cuh"
 
 namespace lmg {
@@ -8,17 +10,40 @@ namespace {
 template <typename R>
 __global__ void k_grid_spill(const Item* __restrict__ items, const int* __restrict__ counters, int item_cap,
                              int W, int RS, int N, const typename Cplx<R>::T* __restrict__ spill,
-                             typename Cplx<R>::T* __restrict__ grid) {
-  // one warp per item slot (the launch covers item_cap slots)
+                             typename Cplx<R>::T* __restrict__ grid, int comp) {
   int nfront;
   const int total = work_total(counters, item_cap, nfront);
-  const int w = static_cast<int>((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
-  if (w < total)
-    spill_item<R>(items, nfront, item_cap, W, RS, N, 32 * cols_per_lane<R>(), spill, grid, w, threadIdx.x & 31);
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += (gridDim.x * blockDim.x) >> 5)
+    spill_item<R>(items, nfront, item_cap, W, RS, N, 32 * cols_per_lane<R>(), spill, grid, w, threadIdx.x & 31,
+                  comp != 0);
 }
 
-void* kernel_for(int W, int dtype, int accum, bool degrid, bool ext) {
-  return ext ? sweep_kernel_ext(W, dtype, accum, degrid) : sweep_kernel_pick<false>(W, dtype, accum, degrid);
+// The parts of cut row pairs, compensated gridding: a warp sums one row of one pair over the
+// pair's parts, their rounding errors apart, and adds the row to the grid once.
+__global__ void k_grid_merge(const Cut* __restrict__ cuts, const int* __restrict__ counters, int part_cap, int W, int N,
+                             const float2* __restrict__ parts, float2* __restrict__ grid) {
+  constexpr int S = strip_width(0);
+  const int lane = threadIdx.x & 31, total = min(counters[kCntCuts], part_cap) * (W + 1);
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += (gridDim.x * blockDim.x) >> 5) {
+    const Cut c = cuts[w / (W + 1)];
+    const int row = w % (W + 1);
+    const float2* p = parts + (static_cast<size_t>(c.part0) * (W + 1) + row) * (2 * S) + 2 * lane;
+    unsigned long long s[2] = {0ull, 0ull}, e[2] = {0ull, 0ull};
+    for (int k = 0; k < c.parts; ++k, p += (W + 1) * 2 * S) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p), r = *reinterpret_cast<const ulonglong2*>(p + S);
+      two_sum_pair(s[0], e[0], v.x);
+      two_sum_pair(s[1], e[1], v.y);
+      e[0] = padd(e[0], r.x);
+      e[1] = padd(e[1], r.y);
+    }
+    float2* dst = grid + static_cast<size_t>((c.r0 + row) % N) * N + c.strip * S + 2 * lane;
+    red_add2(dst, f2unpack(padd(s[0], e[0])), f2unpack(padd(s[1], e[1])));
+  }
+}
+
+void* kernel_for(int W, int dtype, int accum, bool degrid, bool ext, bool direct) {
+  return ext ? sweep_kernel_ext(W, dtype, accum, degrid, direct)
+             : sweep_kernel_pick<false>(W, dtype, accum, degrid, direct);
 }
 
 }  // namespace
@@ -32,15 +57,15 @@ size_t sweep_smem_bytes(int W, int dtype, int Ms, bool table_in_smem, bool degri
   return tab + size_t(warps) * stage_bytes(W, dtype, degrid);
 }
 
-int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext) {
-  void* k = kernel_for(W, dtype, accum, degrid, ext);
+int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct) {
+  void* k = kernel_for(W, dtype, accum, degrid, ext, direct);
   if (!k) return -1;
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_bytes)) == cudaSuccess ? 0 : -1;
 }
 
-int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, int warps,
+int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct, int warps,
                     int* blocks_per_sm) {
-  void* k = kernel_for(W, dtype, accum, degrid, ext);
+  void* k = kernel_for(W, dtype, accum, degrid, ext, direct);
   if (!k) return -1;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, 32 * warps, smem_bytes) == cudaSuccess ? 0
                                                                                                                 : -1;
@@ -63,28 +88,35 @@ int sweep_config(int W, int dtype, int Ms, bool degrid, size_t limit, bool* tabl
 }
 
 int grid_launch(const SweepArgs& a, cudaStream_t st) {
-  void* k = kernel_for(a.W, a.dtype, a.accum, false, a.interp >= 2);
+  void* k = kernel_for(a.W, a.dtype, a.accum, false, a.interp >= 2, a.direct != 0);
   if (!k) return -1;
   const size_t smem = sweep_smem_bytes(a.W, a.dtype, a.Ms, a.table_in_smem != 0, false, a.warps);
   cudaMemsetAsync(a.counters + kCntGridWork, 0, sizeof(int), st);
+  if (a.direct) cudaMemsetAsync(a.grid, 0, size_t(a.N) * size_t(a.N) * (a.dtype ? 16 : 8), st);
   SweepArgs args = a;
   void* params[] = {&args};
   if (cudaLaunchKernel(k, dim3(a.grid_blocks), dim3(32 * a.warps), params, smem, st) != cudaSuccess) return -1;
-  const int spill_blocks = (a.item_cap + 7) / 8;  // 8 warps of 256 threads, one per item slot
-  if (a.dtype) {
-    k_grid_spill<double><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
-                                                       static_cast<const double2*>(a.spill),
-                                                       static_cast<double2*>(a.grid));
-  } else {
-    k_grid_spill<float><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
-                                                      static_cast<const float2*>(a.spill),
-                                                      static_cast<float2*>(a.grid));
+  if (!a.direct) {
+    // a warp per item, 8 warps per CTA, at most 32 CTAs per SM (items beyond that in turn)
+    const int spill_blocks = std::min((a.item_cap + 7) / 8, 32 * kSms);
+    if (a.dtype) {
+      k_grid_spill<double><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
+                                                         static_cast<const double2*>(a.spill),
+                                                         static_cast<double2*>(a.grid), 0);
+    } else {
+      k_grid_spill<float><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
+                                                        static_cast<const float2*>(a.spill),
+                                                        static_cast<float2*>(a.grid), a.accum);
+    }
   }
+  if (a.accum)
+    k_grid_merge<<<2 * kSms, 256, 0, st>>>(a.cuts, a.counters, a.part_cap, a.W, a.N, a.parts,
+                                           static_cast<float2*>(a.grid));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int degrid_launch(const SweepArgs& a, cudaStream_t st, bool zero_out) {
-  void* k = kernel_for(a.W, a.dtype, 0, true, a.interp >= 2);
+  void* k = kernel_for(a.W, a.dtype, 0, true, a.interp >= 2, false);
   if (!k) return -1;
   const size_t smem = sweep_smem_bytes(a.W, a.dtype, a.Ms, a.table_in_smem != 0, true, a.warps);
   // outputs start at zero: each record adds its partial sum (dropped positions stay zero)

@@ -133,6 +133,11 @@ __device__ __forceinline__ void two_sum_pair(unsigned long long& a, unsigned lon
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(lo) : "l"(lo), "l"(ea));
   a = s;
 }
+__device__ __forceinline__ unsigned long long padd(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ unsigned long long pmul(unsigned long long a, unsigned long long b) {
   unsigned long long d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -409,9 +414,10 @@ __device__ __forceinline__ void zero_bytes(unsigned char* p, int bytes, int lane
 }
 
 // Support-start row offsets of an item's row pairs, 32 pairs per block: lane t holds the
-// end offset of pair 32 b + t (the offset of row min(r0 + 2 (32 b + t + 1), r1)).
-__device__ __forceinline__ int pair_ends(const int* __restrict__ off, const Item& item, int b, int lane) {
-  return off[min(item.r0 + 2 * (32 * b + lane + 1), item.r1)];
+// end offset of pair 32 b + t (the offset of row min(r0 + 2 (32 b + t + 1), r1), or the end of
+// the item's records when it holds a part of a pair).
+__device__ __forceinline__ int pair_ends(const int* __restrict__ off, const Item& item, int rend, int b, int lane) {
+  return min(off[min(item.r0 + 2 * (32 * b + lane + 1), item.r1)], rend);
 }
 
 // Lanes L0 .. L1 (inclusive) intersected with [0, 32).
@@ -434,7 +440,10 @@ __device__ __forceinline__ const R* stage_table(const void* table, int n, bool i
   const R* g = static_cast<const R*>(table);
   if (!in_smem) return g;
   R* s = reinterpret_cast<R*>(smem);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s[i] = g[i];
+  // rows are whole 16-byte units (table_stride); the array is 16-byte aligned
+  const int4* g4 = reinterpret_cast<const int4*>(g);
+  int4* s4 = reinterpret_cast<int4*>(smem);
+  for (int i = threadIdx.x; i < n * int(sizeof(R)) / 16; i += blockDim.x) s4[i] = g4[i];
   __syncthreads();
   return s;
 }
@@ -478,6 +487,22 @@ __device__ __forceinline__ void store_cols(typename Cplx<R>::T* dst, const R (&r
       o.x = re[j];
       o.y = im[j];
       dst[j] = o;
+    }
+  }
+}
+// The same added to the grid, one 16-byte reduction where the lane holds anything.
+template <typename R, int KC>
+__device__ __forceinline__ void add_cols(typename Cplx<R>::T* dst, const R (&re)[KC], const R (&im)[KC]) {
+  if constexpr (sizeof(R) == 4 && KC == 2) {
+    if (re[0] != 0.f || im[0] != 0.f || re[1] != 0.f || im[1] != 0.f)
+      red_add2(dst, make_float2(re[0], im[0]), make_float2(re[1], im[1]));
+  } else {
+#pragma unroll
+    for (int j = 0; j < KC; ++j) {
+      typename Cplx<R>::T o;
+      o.x = re[j];
+      o.y = im[j];
+      if (o.x != R(0) || o.y != R(0)) red_add(dst + j, o);
     }
   }
 }
@@ -546,7 +571,9 @@ __device__ __forceinline__ void load_cv_pairs(const unsigned char* s_cv, int l,
 
 // One gridding work item (rows [r0, r1) of one strip), run by the 32 lanes of a warp;
 // `my` is the warp's staging area in shared memory, `tab` the table (shared or global).
-template <int W, typename R, bool COMP, bool EXT = false>
+// DIRECT: the rows are added to a zeroed grid instead of stored, with no spill rows (compiled
+// apart: with both ends in one kernel the 4.1M-visibility sweep took 241 us instead of 224).
+template <int W, typename R, bool COMP, bool EXT = false, bool DIRECT = false>
 __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restrict__ tab, unsigned char* my,
                                           int slot, int lane) {
   using C2 = typename Cplx<R>::T;
@@ -579,6 +606,13 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   const int* __restrict__ off = a.offsets + static_cast<long long>(item.strip) * N;
   const int col0 = item.strip * S + KC * lane;
   const int nrows = item.r1 - item.r0;
+  if (!COMP && item.chain == 0 && item.nrec > 0) return;  // in the chain of an earlier part
+  const bool part = COMP && item.part >= 0;
+  // where the item's rows go: the grid, or for a later chain of a cut pair its spill rows
+  C2* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
+  const bool own = DIRECT || item.own != 0;
+  C2* rows = own ? grid + static_cast<size_t>(item.r0) * N + col0 : sp;
+  const int row_stride = own ? N : S;
   // ring pair h holds relative rows 2h' and 2h' + 1 (h' = h mod RH) of the lane's columns
   P accR[KC][RH], accI[KC][RH];
   P loR[COMP ? KC : 1][COMP ? RH : 1], loI[COMP ? KC : 1][COMP ? RH : 1];
@@ -592,15 +626,28 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
 #pragma unroll
       for (int h = 0; h < RH; ++h) loR[j][h] = loI[j][h] = pzero<P>();
   }
+  // the sums of row d of ring pair h for the lane's columns
+  auto ring_row = [&](int h, int d, R (&orr)[KC], R (&oi)[KC]) {
+#pragma unroll
+    for (int j = 0; j < KC; ++j) {
+      orr[j] = d ? phi(accR[j][h]) : plo(accR[j][h]);
+      oi[j] = d ? phi(accI[j][h]) : plo(accI[j][h]);
+      if constexpr (COMP) {
+        orr[j] += d ? phi(loR[j][h]) : plo(loR[j][h]);
+        oi[j] += d ? phi(loI[j][h]) : plo(loI[j][h]);
+      }
+    }
+  };
   const int myslot = lane & (L::PS - 1);
   zero_bytes(s_cv + 32 * L::CVS * sizeof(R), L::CVS * sizeof(R), lane);
   zero_bytes(s_a + 32 * L::AP, L::AP, lane);
   // software pipeline over 32-record windows of the item (window k = records
   // rb + 32k .. rb + 32k + 31, lane l holding record rb + 32k + l): while window k is
   // processed, the visibilities of window k+1 and the records of window k+2 are in flight
-  const int rb = off[item.r0], rend = off[item.r1];
-  int pend = pair_ends(off, item, 0, lane);
+  const int rb = item.rb, rend = item.rb + (COMP ? item.nrec : item.chain);
+  int pend = pair_ends(off, item, rend, 0, lane);
   int wbase = rb, cstart = rb;
+  int last = -(1 << 20);  // the last group that held records: rows up to last + W + 1 hold sums
   Fetch<R> f0{}, f1{}, f2{};
   fetch_rec(rb, rend, f0);
   fetch_rec(rb + 32, rend, f1);
@@ -613,8 +660,9 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
       const int gb = g0 + gp * kD;
       if (gb < nrows) {
         const int row0 = item.r0 + gb;
-        if (gb > 0 && (gb & 63) == 0) pend = pair_ends(off, item, gb >> 6, lane);
+        if (gb > 0 && (gb & 63) == 0) pend = pair_ends(off, item, rend, gb >> 6, lane);
         const int re = __shfl_sync(0xffffffffu, pend, (gb & 63) >> 1);
+        if (cstart < re) last = gb;
         while (cstart < re) {
           // chunk: records [cstart, ce) of window wbase, staged by lanes cstart - wbase ..
           const int ce = min(re, wbase + 32);
@@ -669,80 +717,121 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
             fetch_rec(wbase + 64, rend, f2);
           }
         }
-        // rows row0 and row0 + 1 (ring pair gp mod RH) are complete: store them, recycle
+        // rows row0 and row0 + 1 (ring pair gp mod RH) are complete: store them (or add them to
+        // the zeroed grid where they hold sums), recycle
         const int h = gp % RH;
+        if (!part && (!DIRECT || gb <= last + W)) {
 #pragma unroll
-        for (int d = 0; d < kD; ++d) {
-          if (gb + d < nrows) {
-            R orr[KC], oi[KC];
-#pragma unroll
-            for (int j = 0; j < KC; ++j) {
-              if constexpr (COMP) {
-                orr[j] = (d ? phi(accR[j][h]) : plo(accR[j][h])) + (d ? phi(loR[j][h]) : plo(loR[j][h]));
-                oi[j] = (d ? phi(accI[j][h]) : plo(accI[j][h])) + (d ? phi(loI[j][h]) : plo(loI[j][h]));
-              } else {
-                orr[j] = d ? phi(accR[j][h]) : plo(accR[j][h]);
-                oi[j] = d ? phi(accI[j][h]) : plo(accI[j][h]);
-              }
+          for (int d = 0; d < kD; ++d) {
+            if (gb + d < nrows) {
+              R orr[KC], oi[KC];
+              ring_row(h, d, orr, oi);
+              C2* dst = rows + static_cast<size_t>(gb + d) * row_stride;
+              if constexpr (DIRECT) add_cols<R, KC>(dst, orr, oi);
+              else store_cols<R, KC>(dst, orr, oi);
             }
-            store_cols<R, KC>(grid + static_cast<size_t>(row0 + d) * N + col0, orr, oi);
           }
         }
+        if (!part) {
 #pragma unroll
-        for (int j = 0; j < KC; ++j) {
-          accR[j][h] = accI[j][h] = pzero<P>();
-          if constexpr (COMP) loR[j][h] = loI[j][h] = pzero<P>();
+          for (int j = 0; j < KC; ++j) {
+            accR[j][h] = accI[j][h] = pzero<P>();
+            if constexpr (COMP) loR[j][h] = loI[j][h] = pzero<P>();
+          }
         }
       }
     }
   }
+  if constexpr (COMP) {
+    if (part) {
+      // a part keeps its sums and their rounding errors apart (k_grid_merge): adding the
+      // parts' rounded sums in float32 would cost the accuracy that compensation buys. The
+      // pair's rows start at zero (stored by its first part).
+      if (!DIRECT && item.own != 0) {
+        const R zero[KC] = {};
+#pragma unroll
+        for (int d = 0; d < kD; ++d) store_cols<R, KC>(rows + static_cast<size_t>(d) * row_stride, zero, zero);
+      }
+      C2* p = a.parts + static_cast<size_t>(item.part) * ((W + 1) * 2 * S) + KC * lane;
+#pragma unroll
+      for (int h = 0; h < RH; ++h) {
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          if (2 * h + d <= W) {
+            R sr[KC], si[KC], er[KC], ei[KC];
+#pragma unroll
+            for (int j = 0; j < KC; ++j) {
+              sr[j] = d ? phi(accR[j][h]) : plo(accR[j][h]);
+              si[j] = d ? phi(accI[j][h]) : plo(accI[j][h]);
+              er[j] = d ? phi(loR[j][h]) : plo(loR[j][h]);
+              ei[j] = d ? phi(loI[j][h]) : plo(loI[j][h]);
+            }
+            store_cols<R, KC>(p + (2 * h + d) * (2 * S), sr, si);
+            store_cols<R, KC>(p + (2 * h + d) * (2 * S) + S, er, ei);
+          }
+        }
+      }
+      return;
+    }
+  }
+  if constexpr (DIRECT) {
+    // ring pair h holds relative rows nrows + ((2h - nrows) mod RS) and the next: add the rows
+    // past the item that hold sums
+#pragma unroll
+    for (int h = 0; h < RH; ++h) {
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {
+        int past = (2 * h + d - nrows) % RS;
+        if (past < 0) past += RS;
+        if (past < W - 1 && nrows + past <= last + W) {
+          R orr[KC], oi[KC];
+          ring_row(h, d, orr, oi);
+          add_cols<R, KC>(grid + static_cast<size_t>((item.r1 + past) % N) * N + col0, orr, oi);
+        }
+      }
+    }
+    return;
+  }
   // spill: ring pair h holds relative rows nrows + ((2h - nrows) mod RS) (and the next);
   // the W - 1 rows after the item carry partial sums
-  C2* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
 #pragma unroll
   for (int h = 0; h < RH; ++h) {
+    if (h == 0 && item.own == 0) continue;
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       R orr[KC], oi[KC];
-#pragma unroll
-      for (int j = 0; j < KC; ++j) {
-        if constexpr (COMP) {
-          orr[j] = (d ? phi(accR[j][h]) : plo(accR[j][h])) + (d ? phi(loR[j][h]) : plo(loR[j][h]));
-          oi[j] = (d ? phi(accI[j][h]) : plo(accI[j][h])) + (d ? phi(loI[j][h]) : plo(loI[j][h]));
-        } else {
-          orr[j] = d ? phi(accR[j][h]) : plo(accR[j][h]);
-          oi[j] = d ? phi(accI[j][h]) : plo(accI[j][h]);
-        }
-      }
+      ring_row(h, d, orr, oi);
       store_cols<R, KC>(sp + static_cast<size_t>(2 * h + d) * S, orr, oi);
     }
   }
 }
 
 // Spill rows of work item w, run by the 32 lanes of a warp after every item stored its own
-// rows: the W - 1 rows past the item (relative rows nrows + j, j < W - 1, held in ring slot
-// (nrows + j) mod RS) are added into the grid. All of them are loaded before the first
-// add, so that the warp waits for one round of loads. S = 32 KC columns, KC per lane.
+// rows: the W - 1 rows past the item (relative rows own + j, held in ring slot (own + j) mod
+// RS), and for the later parts of a cut pair its two rows too (own = 0), are added into the
+// grid. All of them are loaded before the first add, so that the warp waits for one round of
+// loads. S = 32 KC columns, KC per lane.
 template <typename R>
 __device__ __forceinline__ void spill_item(const Item* __restrict__ items, int nfront, int item_cap, int W, int RS,
                                            int N, int S, const typename Cplx<R>::T* __restrict__ spill,
-                                           typename Cplx<R>::T* __restrict__ grid, int w, int lane) {
-  constexpr int kMaxRows = 15;  // W - 1 for W <= 16
+                                           typename Cplx<R>::T* __restrict__ grid, int w, int lane,
+                                           bool comp = false) {  // comp: every part has its own sums
+  constexpr int kMaxRows = 17;  // 2 + W - 1 for W <= 16
   constexpr int KC = cols_per_lane<R>();
   const int slot = item_slot(w, nfront, item_cap);
   const Item item = items[slot];
-  const int nrows = item.r1 - item.r0;
-  if (nrows <= 0 || item.nrec == 0) return;
+  if ((comp ? item.nrec : item.chain) == 0 || (comp && item.part >= 0)) return;
+  const int rows = item.r1 - item.r0 - item.own + W - 1;
   const typename Cplx<R>::T* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
   R vr[kMaxRows][KC], vi[kMaxRows][KC];
 #pragma unroll
   for (int j = 0; j < kMaxRows; ++j)
-    if (j < W - 1) load_cols<R, KC>(sp + static_cast<size_t>((nrows + j) % RS) * S, vr[j], vi[j]);
+    if (j < rows) load_cols<R, KC>(sp + static_cast<size_t>((item.own + j) % RS) * S, vr[j], vi[j]);
   typename Cplx<R>::T* g = grid + static_cast<size_t>(item.strip) * S + KC * lane;
 #pragma unroll
   for (int j = 0; j < kMaxRows; ++j)
-    if (j < W - 1) {
-      typename Cplx<R>::T* dst = g + static_cast<size_t>((item.r1 + j) % N) * N;
+    if (j < rows) {
+      typename Cplx<R>::T* dst = g + static_cast<size_t>((item.r0 + item.own + j) % N) * N;
       if constexpr (sizeof(R) == 4 && KC == 2) {
         red_add2(dst, make_float2(vr[j][0], vi[j][0]), make_float2(vr[j][1], vi[j][1]));
       } else {
@@ -809,8 +898,8 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
   const int myslot = lane & (L::PS - 1);
   zero_bytes(s_cv + 32 * L::CVS * sizeof(R), L::CVS * sizeof(R), lane);
   zero_bytes(s_u + 32 * L::UP, L::UP, lane);
-  const int rb = off[item.r0], rend = off[item.r1];
-  int pend = pair_ends(off, item, 0, lane);
+  const int rb = item.rb, rend = item.rb + item.nrec;
+  int pend = pair_ends(off, item, rend, 0, lane);
   int wbase = rb, cstart = rb;
   int staged = -1;    // window whose records are staged
   unsigned MW = 0u;   // records of that window covering this lane's columns
@@ -825,7 +914,7 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
       if (gb < nrows) {
         put_pair((gp + NPR - 1) % RH);
         fetch_pair(gb + 2 * NPR);
-        if (gb > 0 && (gb & 63) == 0) pend = pair_ends(off, item, gb >> 6, lane);
+        if (gb > 0 && (gb & 63) == 0) pend = pair_ends(off, item, rend, gb >> 6, lane);
         const int re = __shfl_sync(0xffffffffu, pend, (gb & 63) >> 1);
         while (cstart < re) {
           const int ce = min(re, wbase + 32);
@@ -934,7 +1023,7 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
 // Persistent single-plan sweep kernels: each warp takes work items from a counter and runs
 // the per-item sweep. EXT selects the extended lookups (Lagrange, direct calculation),
 // compiled separately so that the nearest / linear kernels keep their register budget.
-template <int W, typename R, bool COMP, bool EXT>
+template <int W, typename R, bool COMP, bool EXT, bool DIRECT>
 __global__ void __launch_bounds__(kThreads, min_blocks<W, R, COMP, EXT>()) k_grid_sweep(const SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -944,7 +1033,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<W, R, COMP, EXT>()) k_gri
   int nfront;
   const int total = work_total(a.counters, a.item_cap, nfront);
   for (int w = next_item(a.counters + kCntGridWork, lane); w < total; w = next_item(a.counters + kCntGridWork, lane))
-    grid_item<W, R, COMP, EXT>(a, tab, my, item_slot(w, nfront, a.item_cap), lane);
+    grid_item<W, R, COMP, EXT, DIRECT>(a, tab, my, item_slot(w, nfront, a.item_cap), lane);
 }
 
 template <int W, typename R, bool EXT>
@@ -963,33 +1052,38 @@ __global__ void __launch_bounds__(kThreads, min_blocks<W, R, false, EXT>()) k_de
   }
 }
 
-template <bool EXT, int W> void* pick_sweep_kernel(int dtype, int accum, bool degrid) {
+template <bool EXT, int W> void* pick_sweep_kernel(int dtype, int accum, bool degrid, bool direct) {
   if (degrid)
     return dtype ? reinterpret_cast<void*>(&k_degrid_sweep<W, double, EXT>)
                  : reinterpret_cast<void*>(&k_degrid_sweep<W, float, EXT>);
-  if (dtype) return reinterpret_cast<void*>(&k_grid_sweep<W, double, false, EXT>);
-  return accum ? reinterpret_cast<void*>(&k_grid_sweep<W, float, true, EXT>)
-               : reinterpret_cast<void*>(&k_grid_sweep<W, float, false, EXT>);
+  if (dtype)
+    return direct ? reinterpret_cast<void*>(&k_grid_sweep<W, double, false, EXT, true>)
+                  : reinterpret_cast<void*>(&k_grid_sweep<W, double, false, EXT, false>);
+  if (accum)
+    return direct ? reinterpret_cast<void*>(&k_grid_sweep<W, float, true, EXT, true>)
+                  : reinterpret_cast<void*>(&k_grid_sweep<W, float, true, EXT, false>);
+  return direct ? reinterpret_cast<void*>(&k_grid_sweep<W, float, false, EXT, true>)
+                : reinterpret_cast<void*>(&k_grid_sweep<W, float, false, EXT, false>);
 }
 
-template <bool EXT> void* sweep_kernel_pick(int W, int dtype, int accum, bool degrid) {
+template <bool EXT> void* sweep_kernel_pick(int W, int dtype, int accum, bool degrid, bool direct) {
   switch (W) {
-    case 1: return pick_sweep_kernel<EXT, 1>(dtype, accum, degrid);
-    case 2: return pick_sweep_kernel<EXT, 2>(dtype, accum, degrid);
-    case 3: return pick_sweep_kernel<EXT, 3>(dtype, accum, degrid);
-    case 4: return pick_sweep_kernel<EXT, 4>(dtype, accum, degrid);
-    case 5: return pick_sweep_kernel<EXT, 5>(dtype, accum, degrid);
-    case 6: return pick_sweep_kernel<EXT, 6>(dtype, accum, degrid);
-    case 7: return pick_sweep_kernel<EXT, 7>(dtype, accum, degrid);
-    case 8: return pick_sweep_kernel<EXT, 8>(dtype, accum, degrid);
-    case 9: return pick_sweep_kernel<EXT, 9>(dtype, accum, degrid);
-    case 10: return pick_sweep_kernel<EXT, 10>(dtype, accum, degrid);
-    case 11: return pick_sweep_kernel<EXT, 11>(dtype, accum, degrid);
-    case 12: return pick_sweep_kernel<EXT, 12>(dtype, accum, degrid);
-    case 13: return pick_sweep_kernel<EXT, 13>(dtype, accum, degrid);
-    case 14: return pick_sweep_kernel<EXT, 14>(dtype, accum, degrid);
-    case 15: return pick_sweep_kernel<EXT, 15>(dtype, accum, degrid);
-    case 16: return pick_sweep_kernel<EXT, 16>(dtype, accum, degrid);
+    case 1: return pick_sweep_kernel<EXT, 1>(dtype, accum, degrid, direct);
+    case 2: return pick_sweep_kernel<EXT, 2>(dtype, accum, degrid, direct);
+    case 3: return pick_sweep_kernel<EXT, 3>(dtype, accum, degrid, direct);
+    case 4: return pick_sweep_kernel<EXT, 4>(dtype, accum, degrid, direct);
+    case 5: return pick_sweep_kernel<EXT, 5>(dtype, accum, degrid, direct);
+    case 6: return pick_sweep_kernel<EXT, 6>(dtype, accum, degrid, direct);
+    case 7: return pick_sweep_kernel<EXT, 7>(dtype, accum, degrid, direct);
+    case 8: return pick_sweep_kernel<EXT, 8>(dtype, accum, degrid, direct);
+    case 9: return pick_sweep_kernel<EXT, 9>(dtype, accum, degrid, direct);
+    case 10: return pick_sweep_kernel<EXT, 10>(dtype, accum, degrid, direct);
+    case 11: return pick_sweep_kernel<EXT, 11>(dtype, accum, degrid, direct);
+    case 12: return pick_sweep_kernel<EXT, 12>(dtype, accum, degrid, direct);
+    case 13: return pick_sweep_kernel<EXT, 13>(dtype, accum, degrid, direct);
+    case 14: return pick_sweep_kernel<EXT, 14>(dtype, accum, degrid, direct);
+    case 15: return pick_sweep_kernel<EXT, 15>(dtype, accum, degrid, direct);
+    case 16: return pick_sweep_kernel<EXT, 16>(dtype, accum, degrid, direct);
     default: return nullptr;
   }
 }
