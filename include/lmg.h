@@ -189,23 +189,24 @@ int lmg_plan_dropped(lmg_plan* p, int64_t* dropped, void* stream);
  *            a float pair updated with an error-free sum)
  *   grid     device complex [N][N]; every cell is overwritten (no pre-zeroing needed)
  * Allocates nothing. Where work items are shorter than W - 1 rows (dense rows), the partial
- * rows of two items are added into the same cells by atomics in either order, so two calls
- * on the same input may differ at the rounding level of the dtype. */
+ * rows of two items are added into the same cells by atomics in either order, and so are the
+ * cells around a strip's edge for LMG_C128: two calls on the same input may differ at the
+ * rounding level of the dtype. */
 int lmg_grid(lmg_plan* p, const void* vis, const void* weights, int accum, void* grid,
              void* stream);
 
 /* lmg_degrid -- V_k = sum_{i,j} C(n_i - u_k) C(m_j - v_k) G[m_j][n_i] (Section 4, the
  * transpose of lmg_grid without weights). grid: device complex [N][N];
  * vis_out: device complex [nvis], every entry overwritten. Allocates nothing. The result
- * is the same bits on every call (each entry is one sum, or two added onto zero when the
- * support crosses a 64-column strip, 32 for complex128). */
+ * is the same bits on every call (each entry is one sum, or for complex64 two added onto
+ * zero when the support crosses a 64-column strip). */
 int lmg_degrid(lmg_plan* p, const void* grid, void* vis_out, void* stream);
 
 /* lmg_degrid_add -- lmg_degrid that adds the predictions to vis_inout instead of
  * overwriting it (Section 4; e.g. the sum of the predictions from several grids, or an
  * output zeroed earlier on another stream). Dropped positions leave their entries as they
- * are. Same arguments, alignment and errors as lmg_degrid. The two adds of a visibility
- * whose support crosses a strip may land in either order. */
+ * are. Same arguments, alignment and errors as lmg_degrid. The two adds of a complex64
+ * visibility whose support crosses a strip may land in either order. */
 int lmg_degrid_add(lmg_plan* p, const void* grid, void* vis_inout, void* stream);
 
 /* lmg_fft -- unnormalised in-place 2-D FFT of a device grid [N][N] in grid index order.
@@ -310,7 +311,8 @@ int lmg_plan_status(lmg_plan* p, int* status_bits, void* stream);
 int lmg_fp32_fma_rate(double* flops_per_s, void* stream);
 
 /* lmg_plan_info -- sizes of a plan: out[0] = N, out[1] = n_image, out[2] = W,
- * out[3] = nvis of the last binning, out[4] = records, out[5] = work items (records and
+ * out[3] = nvis of the last binning, out[4] = records (complex64: a
+ * visibility whose support crosses a strip makes two), out[5] = work items (records and
  * items need a synchronised stream to be current), out[6] = dtype. */
 int lmg_plan_info(lmg_plan* p, int64_t* out, void* stream);
 

@@ -310,7 +310,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   p->n_strips = int(N / strip);
   const size_t rs = dtype == LMG_C128 ? 8 : 4;
   p->Wp = table_stride(p->W, dtype);
-  p->direct = opt.direct && grid_direct(N, dtype);
+  p->direct = dtype == LMG_C128 || (opt.direct && grid_direct(N, dtype));
   p->auto_target = opt.min_item_target == 0;
   p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block,
                                p->auto_target ? item_target_for(max_vis) : opt.min_item_target));
@@ -360,7 +360,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
       (rc = dalloc(reinterpret_cast<unsigned char**>(&p->d_h), h_bytes.size(), "correction")) ||
       (rc = dalloc(&p->hist, size_t(L), "histogram")) ||
       (rc = dalloc(&p->offsets, size_t(L) + 1, "offsets")) || (rc = dalloc(&p->rank, size_t(max_vis), "ranks")) ||
-      (rc = dalloc(&p->partial, size_t(p->nchunks), "scan")) || (rc = dalloc(&p->recs, size_t(2 * max_vis), "records")) ||
+      (rc = dalloc(&p->partial, size_t(p->nchunks), "scan")) || (rc = dalloc(&p->recs, size_t(dtype == LMG_C128 ? max_vis : 2 * max_vis), "records")) ||
       (rc = dalloc(&p->items, size_t(p->item_cap), "items")) || (rc = dalloc(&p->counters, kNumCounters, "counters")) ||
       (!p->direct &&
        (rc = dalloc(reinterpret_cast<unsigned char**>(&p->spill), size_t(p->item_cap) * ring_slots(p->W) * strip * c2, "spill"))) ||
@@ -478,6 +478,7 @@ int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64
                                  : p->item_target;
   a.item_cap = p->item_cap;
   a.skip_empty = p->direct ? 1 : 0;
+  a.one_record = p->dtype == LMG_C128 ? 1 : 0;
   a.cuts = p->cuts;
   a.part_cap = p->part_cap;
   a.max_blocks = p->sms * 8;

@@ -4,8 +4,8 @@
 //
 // Pipeline (all on one stream, no host synchronisation):
 //   1. k_bin_count   per visibility: float64 product to cells, exact fixed-point support
-//                    rule, strip keys (one, or two when the support crosses into the next
-//                    strip); the bucket counter's returned value is the record's rank.
+//                    rule, strip keys (one, or for complex64 two when the support crosses into
+//                    the next strip); the bucket counter's returned value is the record's rank.
 //   2. scan          exclusive prefix sum of the bucket counts (strip-major, row-minor).
 //   3. k_bin_scatter positions recomputed from (u, v) (measured cheaper than storing a
 //                    decoded 16-byte position per visibility and reloading it), records
@@ -58,7 +58,7 @@ __device__ __forceinline__ int next_strip(int strip, int n_strips) { return stri
 // flight together.
 constexpr int kCountIlp = 4;
 
-__global__ void k_bin_count(const double* __restrict__ uv, long long nvis, double scale2, int W,
+__global__ void k_bin_count(const double* __restrict__ uv, long long nvis, double scale2, int W, int Wx,
                             int N, int n_strips, int strip_w, int2* __restrict__ rank, int* __restrict__ hist,
                             int* __restrict__ counters, double2* __restrict__ frac) {
   const int lane = threadIdx.x & 31;  // for the dropped-position count
@@ -82,7 +82,7 @@ __global__ void k_bin_count(const double* __restrict__ uv, long long nvis, doubl
         if (ok) {
           const int strip = strip_of(vp[u].x0, strip_w);
           key1[u] = strip * N + vp[u].y0;
-          if (col_in_strip(vp[u].x0, strip_w) + W > strip_w) key2[u] = next_strip(strip, n_strips) * N + vp[u].y0;
+          if (col_in_strip(vp[u].x0, strip_w) + Wx > strip_w) key2[u] = next_strip(strip, n_strips) * N + vp[u].y0;
         } else {
           bad[u] = true;
         }
@@ -189,7 +189,7 @@ __device__ __forceinline__ int dealt_position(int rho, int n) {
 }
 
 __global__ void k_bin_scatter(const double* __restrict__ uv, double scale2, const int2* __restrict__ rank,
-                              long long nvis, int W, int N, int n_strips, int strip_w,
+                              long long nvis, int W, int Wx, int N, int n_strips, int strip_w,
                               const int* __restrict__ offsets, Rec* __restrict__ recs) {
   // kCountIlp visibilities per thread per iteration: their position, rank and offset loads
   // are in flight together (the pass is bound by its random L2 requests and their latency).
@@ -218,7 +218,7 @@ __global__ void k_bin_scatter(const double* __restrict__ uv, double scale2, cons
         const int strip = strip_of(vp[u].x0, strip_w), xr = col_in_strip(vp[u].x0, strip_w);
         const int pair_row = vp[u].y0 & ~1;
         g1[u] = strip * N + pair_row;
-        if (xr + W > strip_w) g2[u] = next_strip(strip, n_strips) * N + pair_row;
+        if (xr + Wx > strip_w) g2[u] = next_strip(strip, n_strips) * N + pair_row;
       }
     }
     // offsets of the pair's two rows and of the next pair (g is even: one 8-byte load and one
@@ -264,15 +264,15 @@ __global__ void k_bin_scatter(const double* __restrict__ uv, double scale2, cons
 // bins correctly; it only sets the order of the records within a bucket and the cost.
 constexpr int kTrackChunk = 32;
 
-__device__ __forceinline__ void bucket_keys(const VisPos& vp, int W, int N, int n_strips, int strip_w, int& key1,
+__device__ __forceinline__ void bucket_keys(const VisPos& vp, int Wx, int N, int n_strips, int strip_w, int& key1,
                                             int& key2) {
   const int strip = strip_of(vp.x0, strip_w);
   key1 = strip * N + vp.y0;
-  key2 = col_in_strip(vp.x0, strip_w) + W > strip_w ? next_strip(strip, n_strips) * N + vp.y0 : -1;
+  key2 = col_in_strip(vp.x0, strip_w) + Wx > strip_w ? next_strip(strip, n_strips) * N + vp.y0 : -1;
 }
 
 __global__ void k_bin_count_tracks(const double* __restrict__ uv, long long nvis, long long tracks, double scale2,
-                                   int W, int N, int n_strips, int strip_w, int2* __restrict__ rank,
+                                   int W, int Wx, int N, int n_strips, int strip_w, int2* __restrict__ rank,
                                    int* __restrict__ hist, int* __restrict__ counters, double2* __restrict__ frac) {
   const double2* uv2 = reinterpret_cast<const double2*>(uv);
   int* rank1 = reinterpret_cast<int*>(rank);  // rank[k].x = rank1[2 k], rank[k].y = rank1[2 k + 1]
@@ -294,7 +294,7 @@ __global__ void k_bin_count_tracks(const double* __restrict__ uv, long long nvis
       const bool ok = vis_position(uv2[k], scale2, W, N, vp, frac != nullptr ? &dl : nullptr);
       if (frac != nullptr) frac[k] = dl;
       int key1 = -1, key2 = -1;
-      if (ok) bucket_keys(vp, W, N, n_strips, strip_w, key1, key2);
+      if (ok) bucket_keys(vp, Wx, N, n_strips, strip_w, key1, key2);
       else atomicAdd(counters + kCntBad, 1);
       if (key1 != cur1) {
         if (len1 > 0) {
@@ -362,8 +362,8 @@ struct RunPlace {
 };
 
 __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale2, const int2* __restrict__ rank,
-                                     long long nvis, long long tracks, int W, int N, int n_strips, int strip_w,
-                                     const int* __restrict__ offsets, Rec* __restrict__ recs) {
+                                     long long nvis, long long tracks, int W, int Wx, int N, int n_strips,
+                                     int strip_w, const int* __restrict__ offsets, Rec* __restrict__ recs) {
   const double2* uv2 = reinterpret_cast<const double2*>(uv);
   const int* rank1 = reinterpret_cast<const int*>(rank);
   const long long n_t = (nvis + tracks - 1) / tracks;
@@ -378,7 +378,7 @@ __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale
       VisPos vp;
       const bool ok = vis_position(__ldcs(uv2 + k), scale2, W, N, vp);
       int key1 = -1, key2 = -1;
-      if (ok) bucket_keys(vp, W, N, n_strips, strip_w, key1, key2);
+      if (ok) bucket_keys(vp, Wx, N, n_strips, strip_w, key1, key2);
       if (key1 != cur1) {
         cur1 = key1;
         if (key1 >= 0) run1.start(offsets, key1, __ldcs(rank1 + 2 * k));
@@ -531,6 +531,7 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const long long L = static_cast<long long>(a.n_strips) * a.N;
   cudaMemsetAsync(a.hist, 0, sizeof(int) * L, st);
   cudaMemsetAsync(a.counters, 0, sizeof(int) * kNumCounters, st);
+  const int wx = a.one_record ? 1 : a.W;  // columns by which a support crosses into the next strip
   const int threads = 256;
   const long long want_c = (a.nvis + threads * kCountIlp - 1) / (threads * kCountIlp);
   const int blocks_c = static_cast<int>(want_c < a.max_blocks ? (want_c > 0 ? want_c : 1) : a.max_blocks);
@@ -542,19 +543,19 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const long long want_t = (n_tthreads + threads - 1) / threads;
   const int blocks_t = static_cast<int>(want_t < a.max_blocks ? (want_t > 0 ? want_t : 1) : a.max_blocks);
   if (a.tracks > 0)
-    k_bin_count_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.nvis, a.tracks, a.scale2, a.W, a.N, a.n_strips,
+    k_bin_count_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.nvis, a.tracks, a.scale2, a.W, wx, a.N, a.n_strips,
                                                      a.strip, a.rank, a.hist, a.counters, a.frac);
   else
-    k_bin_count<<<blocks_c, threads, 0, st>>>(a.uv, a.nvis, a.scale2, a.W, a.N, a.n_strips, a.strip, a.rank,
+    k_bin_count<<<blocks_c, threads, 0, st>>>(a.uv, a.nvis, a.scale2, a.W, wx, a.N, a.n_strips, a.strip, a.rank,
                                             a.hist, a.counters, a.frac);
   const int nchunks = static_cast<int>((L + kScanChunk - 1) / kScanChunk);
   k_scan_partials<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial);
   k_scan_final<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial, a.offsets);
   if (a.tracks > 0)
-    k_bin_scatter_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.scale2, a.rank, a.nvis, a.tracks, a.W, a.N,
+    k_bin_scatter_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.scale2, a.rank, a.nvis, a.tracks, a.W, wx, a.N,
                                                        a.n_strips, a.strip, a.offsets, a.recs);
   else
-    k_bin_scatter<<<blocks_c, threads, 0, st>>>(a.uv, a.scale2, a.rank, a.nvis, a.W, a.N, a.n_strips, a.strip,
+    k_bin_scatter<<<blocks_c, threads, 0, st>>>(a.uv, a.scale2, a.rank, a.nvis, a.W, wx, a.N, a.n_strips, a.strip,
                                               a.offsets, a.recs);
   const int nblk = (a.N + a.rows_per_block - 1) / a.rows_per_block;
   const int ntask = a.n_strips * nblk;

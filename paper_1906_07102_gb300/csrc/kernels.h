@@ -49,6 +49,7 @@ struct BinArgs {
   long long nvis;
   double scale2;  // N * pixel_scale * 2^32
   int W, N, n_strips, strip;  // strip: columns per strip (strip_width)
+  int one_record;  // a support that crosses into the next strip still makes one record (its strip's)
   int rows_per_block, item_target, item_cap;
   int skip_empty;  // leave out work items without records (gridding into a zeroed grid)
   int max_blocks;
@@ -87,7 +88,7 @@ int part_bound(long long max_vis);
 // item_target_for, raised until item_bound stays within cap items.
 int item_target_within(long long nvis, int n_strips, int N, int rows_per_block, int cap);
 // Gridding by adding into a zeroed grid instead of storing whole rows and adding spill rows:
-// where the grid stays in L2 (129 MB, half of it at most), zeroing and vector reductions cost
+// complex64 where the grid stays in L2 (129 MB, half of it at most; complex128 always), zeroing and vector reductions cost
 // no DRAM traffic, and small items need no spill buffer and no pass over it.
 constexpr bool grid_direct(long long N, int dtype) { return N * N * (dtype ? 16 : 8) <= (48ll << 20); }
 
@@ -134,7 +135,11 @@ int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool d
 int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct, int warps,
                     int* blocks_per_sm);
 // Kernel of the extended lookups (sweep_ext.cu).
-void* sweep_kernel_ext(int W, int dtype, int accum, bool degrid, bool direct);
+void* sweep_kernel_ext(int W, int accum, bool degrid, bool direct);
+// Kernels of complex128 plans (sweep64.cu), their warps per CTA and a warp's shared memory.
+void* sweep64_kernel(int W, bool degrid, bool ext);
+int sweep64_warps();
+size_t sweep64_warp_bytes(int W, bool degrid);
 // Warps per CTA and table placement so that a CTA's shared memory stays within `limit`.
 int sweep_config(int W, int dtype, int Ms, bool degrid, size_t limit, bool* table_in_smem, int* warps);
 

@@ -42,8 +42,9 @@ __global__ void k_grid_merge(const Cut* __restrict__ cuts, const int* __restrict
 }
 
 void* kernel_for(int W, int dtype, int accum, bool degrid, bool ext, bool direct) {
-  return ext ? sweep_kernel_ext(W, dtype, accum, degrid, direct)
-             : sweep_kernel_pick<false>(W, dtype, accum, degrid, direct);
+  if (dtype) return sweep64_kernel(W, degrid, ext);
+  return ext ? sweep_kernel_ext(W, accum, degrid, direct)
+             : sweep_kernel_pick<false>(W, accum, degrid, direct);
 }
 
 }  // namespace
@@ -51,6 +52,7 @@ void* kernel_for(int W, int dtype, int accum, bool degrid, bool ext, bool direct
 int ring_slots(int W) { return kD * ((W + kD - 1 + kD - 1) / kD); }
 
 size_t sweep_smem_bytes(int W, int dtype, int Ms, bool table_in_smem, bool degrid, int warps) {
+  if (dtype) return warps * sweep64_warp_bytes(W, degrid);
   const size_t rs = dtype ? 8 : 4;
   const int Wp = table_stride(W, dtype);
   const size_t tab = table_in_smem ? align16(size_t(Ms + 1) * Wp * rs) : 0;
@@ -72,6 +74,11 @@ int sweep_occupancy(int W, int dtype, int accum, size_t smem_bytes, bool degrid,
 }
 
 int sweep_config(int W, int dtype, int Ms, bool degrid, size_t limit, bool* table_in_smem, int* warps) {
+  if (dtype) {
+    *table_in_smem = false;
+    *warps = sweep64_warps();
+    return 0;
+  }
   const size_t rs = dtype ? 8 : 4;
   const int Wp = table_stride(W, dtype);
   *table_in_smem = align16(size_t(Ms + 1) * Wp * rs) <= 96 * 1024;

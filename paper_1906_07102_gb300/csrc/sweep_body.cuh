@@ -1,6 +1,6 @@
 // Gridding and degridding sweeps (Eqs. 5-6 and their transpose, Section 4): the per-item
 // device code shared by the single-plan kernels (sweep.cu, sweep_ext.cu) and the
-// multi-channel persistent kernels (batch.cu).
+// multi-channel persistent kernels (batch.cu) of complex64 plans (complex128: sweep64_body.cuh).
 //
 // The grid is cut into strips of S = 32 KC columns; a warp owns one work item (a range of
 // rows of one strip) and lane t owns the KC adjacent columns KC t .. KC t + KC - 1 of the
@@ -1052,13 +1052,9 @@ __global__ void __launch_bounds__(kThreads, min_blocks<W, R, false, EXT>()) k_de
   }
 }
 
-template <bool EXT, int W> void* pick_sweep_kernel(int dtype, int accum, bool degrid, bool direct) {
+template <bool EXT, int W> void* pick_sweep_kernel(int accum, bool degrid, bool direct) {
   if (degrid)
-    return dtype ? reinterpret_cast<void*>(&k_degrid_sweep<W, double, EXT>)
-                 : reinterpret_cast<void*>(&k_degrid_sweep<W, float, EXT>);
-  if (dtype)
-    return direct ? reinterpret_cast<void*>(&k_grid_sweep<W, double, false, EXT, true>)
-                  : reinterpret_cast<void*>(&k_grid_sweep<W, double, false, EXT, false>);
+    return reinterpret_cast<void*>(&k_degrid_sweep<W, float, EXT>);
   if (accum)
     return direct ? reinterpret_cast<void*>(&k_grid_sweep<W, float, true, EXT, true>)
                   : reinterpret_cast<void*>(&k_grid_sweep<W, float, true, EXT, false>);
@@ -1066,24 +1062,24 @@ template <bool EXT, int W> void* pick_sweep_kernel(int dtype, int accum, bool de
                 : reinterpret_cast<void*>(&k_grid_sweep<W, float, false, EXT, false>);
 }
 
-template <bool EXT> void* sweep_kernel_pick(int W, int dtype, int accum, bool degrid, bool direct) {
+template <bool EXT> void* sweep_kernel_pick(int W, int accum, bool degrid, bool direct) {
   switch (W) {
-    case 1: return pick_sweep_kernel<EXT, 1>(dtype, accum, degrid, direct);
-    case 2: return pick_sweep_kernel<EXT, 2>(dtype, accum, degrid, direct);
-    case 3: return pick_sweep_kernel<EXT, 3>(dtype, accum, degrid, direct);
-    case 4: return pick_sweep_kernel<EXT, 4>(dtype, accum, degrid, direct);
-    case 5: return pick_sweep_kernel<EXT, 5>(dtype, accum, degrid, direct);
-    case 6: return pick_sweep_kernel<EXT, 6>(dtype, accum, degrid, direct);
-    case 7: return pick_sweep_kernel<EXT, 7>(dtype, accum, degrid, direct);
-    case 8: return pick_sweep_kernel<EXT, 8>(dtype, accum, degrid, direct);
-    case 9: return pick_sweep_kernel<EXT, 9>(dtype, accum, degrid, direct);
-    case 10: return pick_sweep_kernel<EXT, 10>(dtype, accum, degrid, direct);
-    case 11: return pick_sweep_kernel<EXT, 11>(dtype, accum, degrid, direct);
-    case 12: return pick_sweep_kernel<EXT, 12>(dtype, accum, degrid, direct);
-    case 13: return pick_sweep_kernel<EXT, 13>(dtype, accum, degrid, direct);
-    case 14: return pick_sweep_kernel<EXT, 14>(dtype, accum, degrid, direct);
-    case 15: return pick_sweep_kernel<EXT, 15>(dtype, accum, degrid, direct);
-    case 16: return pick_sweep_kernel<EXT, 16>(dtype, accum, degrid, direct);
+    case 1: return pick_sweep_kernel<EXT, 1>(accum, degrid, direct);
+    case 2: return pick_sweep_kernel<EXT, 2>(accum, degrid, direct);
+    case 3: return pick_sweep_kernel<EXT, 3>(accum, degrid, direct);
+    case 4: return pick_sweep_kernel<EXT, 4>(accum, degrid, direct);
+    case 5: return pick_sweep_kernel<EXT, 5>(accum, degrid, direct);
+    case 6: return pick_sweep_kernel<EXT, 6>(accum, degrid, direct);
+    case 7: return pick_sweep_kernel<EXT, 7>(accum, degrid, direct);
+    case 8: return pick_sweep_kernel<EXT, 8>(accum, degrid, direct);
+    case 9: return pick_sweep_kernel<EXT, 9>(accum, degrid, direct);
+    case 10: return pick_sweep_kernel<EXT, 10>(accum, degrid, direct);
+    case 11: return pick_sweep_kernel<EXT, 11>(accum, degrid, direct);
+    case 12: return pick_sweep_kernel<EXT, 12>(accum, degrid, direct);
+    case 13: return pick_sweep_kernel<EXT, 13>(accum, degrid, direct);
+    case 14: return pick_sweep_kernel<EXT, 14>(accum, degrid, direct);
+    case 15: return pick_sweep_kernel<EXT, 15>(accum, degrid, direct);
+    case 16: return pick_sweep_kernel<EXT, 16>(accum, degrid, direct);
     default: return nullptr;
   }
 }

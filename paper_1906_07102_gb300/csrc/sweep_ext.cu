@@ -5,8 +5,8 @@
 
 namespace lmg {
 
-void* sweep_kernel_ext(int W, int dtype, int accum, bool degrid, bool direct) {
-  return sweep_kernel_pick<true>(W, dtype, accum, degrid, direct);
+void* sweep_kernel_ext(int W, int accum, bool degrid, bool direct) {
+  return sweep_kernel_pick<true>(W, accum, degrid, direct);
 }
 
 }  // namespace lmg
