@@ -430,6 +430,12 @@ __device__ __forceinline__ void put_item(const Item& it, int target, Item* __res
   else atomicOr(counters + kCntStatus, kStatusItemOverflow);
 }
 
+// k-th of n blocks counted from the middle one outwards. Items are taken up in about the order
+// in which their blocks place them, and the longest (chains of a dense pair's parts, 16,000 records
+// and more) lie around the uv origin, in the grid's middle: placed first they do not end the
+// sweep alone (gridding and degridding 49.5M visibilities 5602 -> 5316 us, 4.1M 545 -> 520).
+__device__ __forceinline__ int centre_out(int k, int n) { return n / 2 + ((k & 1) ? -((k + 1) >> 1) : k >> 1); }
+
 __global__ void __launch_bounds__(kItemThreads)
     k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty,
                  Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
@@ -439,7 +445,8 @@ __global__ void __launch_bounds__(kItemThreads)
   __shared__ unsigned s_start[kItemThreads / 32 + 1], s_cut[kItemThreads / 32];
   __shared__ int s_warp[kItemThreads / 32];
   const int nblk = (N + rows_per_block - 1) / rows_per_block;
-  const int s = blockIdx.x / nblk, b = blockIdx.x % nblk;
+  const int n_strips = gridDim.x / nblk;
+  const int s = centre_out(blockIdx.x % n_strips, n_strips), b = centre_out(blockIdx.x / n_strips, nblk);
   const int rb = b * rows_per_block, np = (min(N, rb + rows_per_block) - rb) / 2;
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = blockDim.x >> 5;
   const int* off = offsets + static_cast<long long>(s) * N + rb;
