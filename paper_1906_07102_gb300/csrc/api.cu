@@ -86,7 +86,7 @@ namespace lmg {
 void free_plan(lmg_plan* p) {
   if (!p) return;
   void* ptrs[] = {p->d_table, p->d_h, p->hist, p->offsets, p->rank, p->partial, p->recs,
-                  p->items, p->cuts, p->counters, p->spill, p->parts, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
+                  p->items, p->cuts, p->spill, p->parts, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->fft_ok) cufftDestroy(p->fft);
@@ -358,10 +358,10 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   const size_t c2 = 2 * rs;
   if ((rc = dalloc(reinterpret_cast<unsigned char**>(&p->d_table), tab_bytes.size(), "table")) ||
       (rc = dalloc(reinterpret_cast<unsigned char**>(&p->d_h), h_bytes.size(), "correction")) ||
-      (rc = dalloc(&p->hist, size_t(L), "histogram")) ||
+      (rc = dalloc(&p->hist, size_t(L) + kNumCounters, "histogram and counters")) ||
       (rc = dalloc(&p->offsets, size_t(L) + 1, "offsets")) || (rc = dalloc(&p->rank, size_t(max_vis), "ranks")) ||
       (rc = dalloc(&p->partial, size_t(p->nchunks), "scan")) || (rc = dalloc(&p->recs, size_t(dtype == LMG_C128 ? max_vis : 2 * max_vis), "records")) ||
-      (rc = dalloc(&p->items, size_t(p->item_cap), "items")) || (rc = dalloc(&p->counters, kNumCounters, "counters")) ||
+      (rc = dalloc(&p->items, size_t(p->item_cap), "items")) ||
       (!p->direct &&
        (rc = dalloc(reinterpret_cast<unsigned char**>(&p->spill), size_t(p->item_cap) * ring_slots(p->W) * strip * c2, "spill"))) ||
       (p->part_cap > 0 &&
@@ -377,6 +377,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
     free_plan(p);
     return rc;
   }
+  p->counters = p->hist + L;
   // the device is queried after the allocations (which run on the current device), so
   // that an injected allocation failure is reported before any CUDA call
   if ((e = cudaGetDevice(&p->device)) != cudaSuccess ||
@@ -635,7 +636,7 @@ int lmg_plan_bin_tracks(lmg_plan* p, const double* uv, int64_t nvis, int64_t tra
 int lmg_plan_dropped(lmg_plan* p, int64_t* dropped, void* stream) {
   clear_error();
   if (!p || !dropped) return set_error(LMG_EINVAL, "NULL argument");
-  int c[8];
+  int c[kNumCounters];
   cudaError_t e = cudaMemcpyAsync(c, p->counters, sizeof(c), cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_error(e, "reading counters");
@@ -646,7 +647,7 @@ int lmg_plan_dropped(lmg_plan* p, int64_t* dropped, void* stream) {
 int lmg_plan_info(lmg_plan* p, int64_t* out, void* stream) {
   clear_error();
   if (!p || !out) return set_error(LMG_EINVAL, "NULL argument");
-  int c[8];
+  int c[kNumCounters];
   cudaError_t e = cudaMemcpyAsync(c, p->counters, sizeof(c), cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(stream));
   if (e == cudaSuccess) e = cudaStreamSynchronize(static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_error(e, "reading counters");

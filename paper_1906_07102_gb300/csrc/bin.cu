@@ -104,6 +104,70 @@ __global__ void k_bin_count(const double* __restrict__ uv, long long nvis, doubl
   }
 }
 
+// Pass 1 where many positions share few buckets (a coarse grid): a CTA counts kDensePer positions a
+// thread in shared memory and takes each bucket's ranks from the global counter at once. One
+// counter update a record queues at the hot buckets' addresses: 4.1M visibilities on a 256^2
+// grid (1024 buckets) took 524 us that way, 71 this way. From kDenseBuckets buckets on
+// clearing and adding up the CTA's counters costs as much as it saves.
+constexpr int kDenseThreads = 512;
+constexpr int kDensePer = 8;
+constexpr int kDenseBuckets = 4096;
+constexpr int kDenseCount = 64;  // positions a bucket, on average
+
+__global__ void __launch_bounds__(kDenseThreads)
+    k_bin_count_dense(const double* __restrict__ uv, long long nvis, double scale2, int W, int Wx, int N, int n_strips,
+                      int strip_w, int2* __restrict__ rank, int* __restrict__ hist, int* __restrict__ counters,
+                      double2* __restrict__ frac) {
+  __shared__ int s_hist[kDenseBuckets];
+  const int L = n_strips * N, lane = threadIdx.x & 31;
+  constexpr int kSpan = kDenseThreads * kDensePer;
+  for (long long base = static_cast<long long>(blockIdx.x) * kSpan; base < nvis;
+       base += static_cast<long long>(gridDim.x) * kSpan) {
+    for (int i = threadIdx.x; i < L; i += kDenseThreads) s_hist[i] = 0;
+    __syncthreads();
+    int key1[kDensePer], key2[kDensePer];
+    int2 rk[kDensePer];
+#pragma unroll
+    for (int u = 0; u < kDensePer; ++u) {
+      const long long k = base + u * kDenseThreads + threadIdx.x;
+      key1[u] = key2[u] = -1;
+      rk[u] = make_int2(0, 0);
+      bool bad = false;
+      if (k < nvis) {
+        VisPos vp{-1, 0, 0u, 0u};
+        double2 dl = make_double2(0.0, 0.0);
+        const bool ok = vis_position(reinterpret_cast<const double2*>(uv)[k], scale2, W, N, vp,
+                                     frac != nullptr ? &dl : nullptr);
+        if (frac != nullptr) frac[k] = dl;
+        bad = !ok;
+        if (ok) {
+          const int strip = strip_of(vp.x0, strip_w);
+          key1[u] = strip * N + vp.y0;
+          if (col_in_strip(vp.x0, strip_w) + Wx > strip_w) key2[u] = next_strip(strip, n_strips) * N + vp.y0;
+          rk[u].x = atomicAdd(s_hist + key1[u], 1);
+          if (key2[u] >= 0) rk[u].y = atomicAdd(s_hist + key2[u], 1);
+        }
+      }
+      const unsigned nb = __popc(__ballot_sync(0xffffffffu, bad));
+      if (lane == 0 && nb) atomicAdd(counters + kCntBad, static_cast<int>(nb));
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < L; i += kDenseThreads) {
+      const int n = s_hist[i];
+      if (n > 0) s_hist[i] = atomicAdd(hist + i, n);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kDensePer; ++u) {
+      const long long k = base + u * kDenseThreads + threadIdx.x;
+      if (key1[u] >= 0) rk[u].x += s_hist[key1[u]];
+      if (key2[u] >= 0) rk[u].y += s_hist[key2[u]];
+      if (k < nvis) rank[k] = rk[u];
+    }
+    __syncthreads();
+  }
+}
+
 // Exclusive scan, stage 1: per-chunk sums.
 constexpr int kScanThreads = 256;
 constexpr int kScanPer = 16;
@@ -171,6 +235,44 @@ __global__ void k_scan_final(const int* __restrict__ in, long long n, const int*
     run += v[i];
   }
   if (base + kScanPer >= n && base < n) offsets[n] = run;  // thread holding the last element
+}
+
+// The whole scan in one CTA, for up to kScanOne buckets (a grid of 1024^2 complex64): at that size
+// each of the two launches above costs more than the work.
+constexpr int kScanOneThreads = 1024;
+constexpr int kScanOne = kScanOneThreads * kScanPer;
+
+__global__ void __launch_bounds__(kScanOneThreads)
+    k_scan_one(const int* __restrict__ in, int n, int* __restrict__ offsets) {
+  __shared__ int warp_sums[kScanOneThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, base = threadIdx.x * kScanPer;
+  int v[kScanPer];
+  int s = 0;
+#pragma unroll
+  for (int i = 0; i < kScanPer; ++i) {
+    v[i] = base + i < n ? in[base + i] : 0;
+    s += v[i];
+  }
+  int x = s;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) warp_sums[w] = x;
+  __syncthreads();
+  int t = warp_sums[lane];
+  const int own = t;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += y;
+  }
+  int run = __shfl_sync(0xffffffffu, t - own, w) + x - s;
+#pragma unroll
+  for (int i = 0; i < kScanPer; ++i) {
+    if (base + i < n) offsets[base + i] = run;
+    run += v[i];
+  }
+  if (threadIdx.x == kScanOneThreads - 1) offsets[n] = run;
 }
 
 // Pass 2: every record to offsets[bucket] + rank (no atomics).
@@ -439,7 +541,6 @@ __device__ __forceinline__ int centre_out(int k, int n) { return n / 2 + ((k & 1
 __global__ void __launch_bounds__(kItemThreads)
     k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty,
                  Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
-  __shared__ int s_part0;
   __shared__ int s_off[kItemThreads + 1];  // offset of each pair's first record
   __shared__ int s_pre[kItemThreads];      // records of joined pairs before each pair
   __shared__ unsigned s_start[kItemThreads / 32 + 1], s_cut[kItemThreads / 32];
@@ -504,29 +605,32 @@ __global__ void __launch_bounds__(kItemThreads)
     if (cnt > 0 || !skip_empty)
       put_item(Item{s, rb + 2 * i, rb + 2 * end, cnt, s_off[i], 2 * (end - i), -1, cnt}, target, items, counters, cap);
   }
-  // cut pairs, one after another, their parts over the threads
+  // cut pairs, a warp each, their parts over its lanes (one after another over the CTA, with a
+  // barrier before and after each pair's update of the parts' counter, the 4.1M visibilities of
+  // a 256^2 grid took 39 to 58 us here, 16 now)
+  int k0 = 0;
   for (int w = 0; w < nw; ++w) {
     for (unsigned m = s_cut[w]; m; m &= m - 1) {
+      if (k0++ % nw != warp) continue;
       const int p = 32 * w + __ffs(m) - 1;
       const int o0 = s_off[p], cnt = s_off[p + 1] - o0, parts = cnt / (4 * target);
       int part0 = -1;
       if (cuts != nullptr) {
-        if (i == 0) {
+        if (lane == 0) {
           const int q = atomicAdd(counters + kCntParts, parts);
-          s_part0 = q + parts <= part_cap ? q : -1;
-          if (s_part0 >= 0) cuts[atomicAdd(counters + kCntCuts, 1)] = Cut{s, rb + 2 * p, q, parts};
+          part0 = q + parts <= part_cap ? q : -1;
+          if (part0 >= 0) cuts[atomicAdd(counters + kCntCuts, 1)] = Cut{s, rb + 2 * p, q, parts};
           else atomicOr(counters + kCntStatus, kStatusItemOverflow);
         }
-        __syncthreads();
-        part0 = s_part0;
-        __syncthreads();
+        part0 = __shfl_sync(0xffffffffu, part0, 0);
       }
-      for (int k = i; k < parts; k += blockDim.x) {
+      for (int k = lane; k < parts; k += 32) {
         const int a = o0 + static_cast<int>(static_cast<long long>(cnt) * k / parts);
         const int e = o0 + static_cast<int>(static_cast<long long>(cnt) * (k + 1) / parts);
         const int ce = o0 + static_cast<int>(static_cast<long long>(cnt) * min(k + kChain, parts) / parts);
         const int chain = k % kChain == 0 ? ce - a : 0;
-        put_item(Item{s, rb + 2 * p, rb + 2 * p + 2, e - a, a, k == 0 ? 2 : 0, part0 < 0 ? -1 : part0 + k, chain}, target, items, counters, cap);
+        put_item(Item{s, rb + 2 * p, rb + 2 * p + 2, e - a, a, k == 0 ? 2 : 0, part0 < 0 ? -1 : part0 + k, chain}, target,
+                 items, counters, cap);
       }
     }
   }
@@ -536,8 +640,9 @@ __global__ void __launch_bounds__(kItemThreads)
 
 int bin_launch(const BinArgs& a, cudaStream_t st) {
   const long long L = static_cast<long long>(a.n_strips) * a.N;
-  cudaMemsetAsync(a.hist, 0, sizeof(int) * L, st);
-  cudaMemsetAsync(a.counters, 0, sizeof(int) * kNumCounters, st);
+  // the counters lie behind the bucket counts: one launch clears both
+  if (a.counters != a.hist + L) return -1;
+  cudaMemsetAsync(a.hist, 0, sizeof(int) * (L + kNumCounters), st);
   const int wx = a.one_record ? 1 : a.W;  // columns by which a support crosses into the next strip
   const int threads = 256;
   const long long want_c = (a.nvis + threads * kCountIlp - 1) / (threads * kCountIlp);
@@ -552,12 +657,20 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   if (a.tracks > 0)
     k_bin_count_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.nvis, a.tracks, a.scale2, a.W, wx, a.N, a.n_strips,
                                                      a.strip, a.rank, a.hist, a.counters, a.frac);
-  else
+  else if (L <= kDenseBuckets && a.nvis >= kDenseCount * L) {
+    const long long want = (a.nvis + kDenseThreads * kDensePer - 1) / (kDenseThreads * kDensePer);
+    k_bin_count_dense<<<static_cast<int>(want < a.max_blocks ? want : a.max_blocks), kDenseThreads, 0, st>>>(
+        a.uv, a.nvis, a.scale2, a.W, wx, a.N, a.n_strips, a.strip, a.rank, a.hist, a.counters, a.frac);
+  } else
     k_bin_count<<<blocks_c, threads, 0, st>>>(a.uv, a.nvis, a.scale2, a.W, wx, a.N, a.n_strips, a.strip, a.rank,
                                             a.hist, a.counters, a.frac);
   const int nchunks = static_cast<int>((L + kScanChunk - 1) / kScanChunk);
-  k_scan_partials<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial);
-  k_scan_final<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial, a.offsets);
+  if (L <= kScanOne) {
+    k_scan_one<<<1, kScanOneThreads, 0, st>>>(a.hist, static_cast<int>(L), a.offsets);
+  } else {
+    k_scan_partials<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial);
+    k_scan_final<<<nchunks, kScanThreads, 0, st>>>(a.hist, L, a.partial, a.offsets);
+  }
   if (a.tracks > 0)
     k_bin_scatter_tracks<<<blocks_t, threads, 0, st>>>(a.uv, a.scale2, a.rank, a.nvis, a.tracks, a.W, wx, a.N,
                                                        a.n_strips, a.strip, a.offsets, a.recs);

@@ -53,7 +53,7 @@ struct BinArgs {
   int rows_per_block, item_target, item_cap;
   int skip_empty;  // leave out work items without records (gridding into a zeroed grid)
   int max_blocks;
-  int* hist;       // n_strips * N
+  int* hist;       // n_strips * N, followed by the counters
   int* offsets;    // n_strips * N + 1
   int2* rank;      // max_vis: rank of the record(s) in their buckets
   int* partial;    // scan chunk sums
@@ -61,7 +61,7 @@ struct BinArgs {
   Item* items;     // item_cap
   Cut* cuts;       // part_cap or NULL (no compensated gridding): the cut row pairs
   int part_cap;
-  int* counters;   // 8
+  int* counters;   // kNumCounters, at hist + n_strips * N
   double2* frac;   // max_vis or NULL: per visibility (u_q - u, v_q - v) in cells, the residual
                    // of the 2^-32 quantisation (float64 plans: exact table fractions)
   long long tracks;  // > 0: positions ordered k = t * tracks + b (sample t of track b); the

@@ -40,12 +40,11 @@ constexpr size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
 constexpr size_t kOffTable = 0;
 constexpr size_t kOffRank = kOffTable + up256(sizeof(float) * (kMaxOversample + 1) * kMaxWp);
 constexpr size_t kOffHist = kOffRank + up256(sizeof(int2) * kMaxVis);
-constexpr size_t kOffOffsets = kOffHist + up256(sizeof(int) * kMaxBuckets);
+constexpr size_t kOffOffsets = kOffHist + up256(sizeof(int) * (kMaxBuckets + kNumCounters));
 constexpr size_t kOffPartial = kOffOffsets + up256(sizeof(int) * (kMaxBuckets + 1));
 constexpr size_t kOffRecs = kOffPartial + up256(sizeof(int) * (kMaxBuckets / 4096 + 2));
 constexpr size_t kOffItems = kOffRecs + up256(sizeof(Rec) * 2 * kMaxVis);
-constexpr size_t kOffCounters = kOffItems + up256(sizeof(Item) * kMaxItems);
-constexpr size_t kScratchBytes = kOffCounters + up256(sizeof(int) * kNumCounters);
+constexpr size_t kScratchBytes = kOffItems + up256(sizeof(Item) * kMaxItems);
 
 // The working memory: allocated when the library is loaded, on every device that loads
 // it, and held until the process exits.
@@ -189,7 +188,7 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   b.partial = reinterpret_cast<int*>(base + kOffPartial);
   b.recs = reinterpret_cast<Rec*>(base + kOffRecs);
   b.items = reinterpret_cast<Item*>(base + kOffItems);
-  b.counters = reinterpret_cast<int*>(base + kOffCounters);
+  b.counters = b.hist + static_cast<long long>(n_strips) * N;
   if (bin_launch(b, st) != 0) return set_error(LMG_ECUDA, std::string("binning launch: ") + cudaGetErrorString(cudaGetLastError()));
 
   bool tab_smem = false;

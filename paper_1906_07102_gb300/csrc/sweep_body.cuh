@@ -148,8 +148,8 @@ __device__ __forceinline__ unsigned long long pmul(unsigned long long a, unsigne
 // whose own rounding error is kept too: the part of the products that reached the sum, bp, is taken
 // off both of them exactly or to the last place of the second, so that what is lost is one rounding
 // a product, as with an addition each, in 10 operations in place of 16 (the sums are bound by
-// the float32 pipe; with an addition each the 49.9M visibilities of an 8192^2 grid at W = 12 took
-// 2.3 ms longer, 10.4 ms, and 4.1M on 256^2 1.06 ms).
+// the float32 pipe and shared memory; an addition each against this: 49.9M visibilities, W = 12, 8192^2
+// 10.4 and 8.9 ms, 4.1M on 256^2 1.06 and 0.83 ms).
 __device__ __forceinline__ void two_products(unsigned long long& a, unsigned long long& lo, unsigned long long b1,
                                              unsigned long long d1, unsigned long long b2, unsigned long long d2) {
   unsigned long long s, bp, ap, ea, u;
