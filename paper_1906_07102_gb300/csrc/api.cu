@@ -313,7 +313,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   p->direct = dtype == LMG_C128 || (opt.direct && grid_direct(N, dtype));
   p->auto_target = opt.min_item_target == 0;
   p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block,
-                               p->auto_target ? item_target_for(max_vis) : opt.min_item_target));
+                               p->auto_target ? item_target_for(max_vis, dtype) : opt.min_item_target));
   p->part_cap = dtype == LMG_C64 && p->auto_target ? part_bound(max_vis) : 0;
   if (inject_fault("item_cap")) p->item_cap = 1;
   const long long L = (long long)p->n_strips * N;
@@ -475,7 +475,7 @@ int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64
   a.n_strips = p->n_strips;
   a.strip = p->strip;
   a.rows_per_block = p->rows_per_block;
-  a.item_target = p->auto_target ? item_target_within(nvis, p->n_strips, int(p->N), p->rows_per_block, p->item_cap)
+  a.item_target = p->auto_target ? item_target_within(nvis, p->dtype, p->n_strips, int(p->N), p->rows_per_block, p->item_cap)
                                  : p->item_target;
   a.item_cap = p->item_cap;
   a.skip_empty = p->direct ? 1 : 0;

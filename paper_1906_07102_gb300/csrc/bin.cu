@@ -507,6 +507,9 @@ __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale
 // is otherwise a serial chain that the whole launch waits for (4.1M visibilities on a 256^2 grid:
 // 512 such items kept a fifth of the resident warps busy, and degridding took 4.4 ms, 0.43 with
 // the cut).
+// fine (complex128): items are cut at any pair, and a pair of 2 target records or more into parts of
+// one to two targets: those sweeps end in tails of long items (see item_target_for), and their sums
+// meet at the strips' edges in any order anyway.
 // Items per block are at most 1 + count / target: a cut pair of n >= 8 target records gives at
 // most n / (4 target) parts and one more boundary between joined pairs.
 // Items with more than target/2 records are placed from the front of the array and the others
@@ -539,7 +542,7 @@ __device__ __forceinline__ void put_item(const Item& it, int target, Item* __res
 __device__ __forceinline__ int centre_out(int k, int n) { return n / 2 + ((k & 1) ? -((k + 1) >> 1) : k >> 1); }
 
 __global__ void __launch_bounds__(kItemThreads)
-    k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty,
+    k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty, int fine,
                  Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
   __shared__ int s_off[kItemThreads + 1];  // offset of each pair's first record
   __shared__ int s_pre[kItemThreads];      // records of joined pairs before each pair
@@ -554,7 +557,7 @@ __global__ void __launch_bounds__(kItemThreads)
   for (int k = i; k <= np; k += blockDim.x) s_off[k] = off[2 * k];
   __syncthreads();
   // unit of pair i: u pairs, the last unit of the block with the remainder
-  const int u = target < kDenseUnit ? max(1, W >> 1) : 1, nu = max(1, np / u);
+  const int u = target < kDenseUnit && !fine ? max(1, W >> 1) : 1, nu = max(1, np / u);
   auto unit_first = [&](int k) { return min(k / u, nu - 1) * u; };
   auto dense_unit = [&](int first) {
     const int end = first / u == nu - 1 ? np : first + u;
@@ -564,7 +567,8 @@ __global__ void __launch_bounds__(kItemThreads)
   const int first = in ? unit_first(i) : 0;
   const bool dense = in && dense_unit(first);
   const int n = in ? s_off[i + 1] - s_off[i] : 0;
-  const bool cut = dense && n >= 8 * target;
+  const int part = fine ? target : 4 * target;  // records of a cut pair's part, about
+  const bool cut = dense && n >= 2 * part;
   const int nj = cut ? 0 : n;
   int x = nj;
   for (int o = 1; o < 32; o <<= 1) {
@@ -613,7 +617,7 @@ __global__ void __launch_bounds__(kItemThreads)
     for (unsigned m = s_cut[w]; m; m &= m - 1) {
       if (k0++ % nw != warp) continue;
       const int p = 32 * w + __ffs(m) - 1;
-      const int o0 = s_off[p], cnt = s_off[p + 1] - o0, parts = cnt / (4 * target);
+      const int o0 = s_off[p], cnt = s_off[p + 1] - o0, parts = cnt / part;
       int part0 = -1;
       if (cuts != nullptr) {
         if (lane == 0) {
@@ -681,7 +685,8 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const int ntask = a.n_strips * nblk;
   if (a.rows_per_block > kMaxRowsPerBlock) return -1;
   const int item_threads = a.rows_per_block <= 256 ? 128 : kItemThreads;
-  k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty, a.items,
+  k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty,
+                                               a.one_record, a.items,
                                                a.counters, a.item_cap, a.cuts, a.part_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -691,8 +696,12 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
 // 2432 resident warps and the sweep took 50 us, as long as one item does. 32 warps per SM give
 // each warp about two items; from 32 records down an item is all start-up (its grid rows and
 // offsets); above 512 nothing is gained (best of {256 .. 2048} on 4.1M-visibility tracks).
-int item_target_for(long long nvis) {
-  const long long t = nvis / (32 * kSms);
+// complex128: 96 items per SM, of which 10 to 32 are swept at a time. A record costs its SM 325
+// cycles at W = 14, an item's rows little beside it: with 32 items per SM, two to three a warp, the
+// float64 pipe stood still for a sixth of the sweep. Gridding and degridding in us: 1.03M visibilities,
+// W = 14 cubic, 2048^2: 1646 + 1666 -> 1311 + 1320; 0.40M, W = 9, 256^2: 644 + 653 -> 275 + 277.
+int item_target_for(long long nvis, int dtype) {
+  const long long t = nvis / ((dtype ? 96 : 32) * kSms);
   return static_cast<int>(t < 32 ? 32 : (t > 512 ? 512 : t));
 }
 
@@ -702,17 +711,17 @@ long long item_bound(long long nvis, int n_strips, int N, int rows_per_block, in
   return n_strips * nblk + 2 * nvis / target + 2;
 }
 
-// A cut pair's n records give at most n / (4 target) parts, and nvis positions two records
-// each; nvis / item_target_for(nvis) is largest at max_vis or where the target passes 33.
+// Complex64: a cut pair's n records give at most n / (4 target) parts, and nvis positions two records
+// each; nvis / item_target_for(nvis, 0) is largest at max_vis or where the target passes 33.
 int part_bound(long long max_vis) {
   const long long n = max_vis / 32 <= 32 * kSms ? max_vis / 32 : 33 * kSms;
   return static_cast<int>((n > max_vis / 512 ? n : max_vis / 512) / 2 + 1);
 }
 
-int item_target_within(long long nvis, int n_strips, int N, int rows_per_block, int cap) {
+int item_target_within(long long nvis, int dtype, int n_strips, int N, int rows_per_block, int cap) {
   const long long room = cap - item_bound(0, n_strips, N, rows_per_block, 1);
   const long long least = room > 0 ? (2 * nvis + room - 1) / room : 0;
-  const int t = item_target_for(nvis);
+  const int t = item_target_for(nvis, dtype);
   return least > t ? static_cast<int>(least) : t;
 }
 

@@ -81,12 +81,12 @@ int xform_model_launch(const void* image, void* grid, void* scratch, const float
 
 int bin_launch(const BinArgs& a, cudaStream_t st);
 int bin_scan_chunks(long long L);
-int item_target_for(long long nvis);
+int item_target_for(long long nvis, int dtype);
 long long item_bound(long long nvis, int n_strips, int N, int rows_per_block, int target);
 // Parts of cut row pairs that up to max_vis positions can make.
 int part_bound(long long max_vis);
 // item_target_for, raised until item_bound stays within cap items.
-int item_target_within(long long nvis, int n_strips, int N, int rows_per_block, int cap);
+int item_target_within(long long nvis, int dtype, int n_strips, int N, int rows_per_block, int cap);
 // Gridding by adding into a zeroed grid instead of storing whole rows and adding spill rows:
 // complex64 where the grid stays in L2 (129 MB, half of it at most; complex128 always), zeroing and vector reductions cost
 // no DRAM traffic, and small items need no spill buffer and no pass over it.

@@ -178,7 +178,7 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   b.n_strips = n_strips;
   b.strip = kStaticStrip;
   b.rows_per_block = kRowsPerBlock;
-  b.item_target = item_target_within(nvis, n_strips, int(N), kRowsPerBlock, item_cap);
+  b.item_target = item_target_within(nvis, LMG_C64, n_strips, int(N), kRowsPerBlock, item_cap);
   b.item_cap = item_cap;
   b.skip_empty = 1;
   b.max_blocks = s->sms * 8;

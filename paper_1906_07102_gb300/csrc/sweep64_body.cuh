@@ -18,10 +18,10 @@
 //   * degridding: lane g W + c sums column c over the rows g, g + G, .. (G = min(32 / W, W)), and
 //     four lanes add up a record's partial sums, weighted by Cu.
 // Measured against the float32 sweeps' scheme in float64 (one column a lane, ring in registers),
-// gridding and degridding in us: 1.03M visibilities, W = 14 cubic, 2048^2: 3194 + 3017 -> 1646 + 1666;
-// 0.81M, W = 7 linear, 2048^2: 726 + 827 -> 442 + 539; 0.40M, W = 9, 256^2: 2450 + 2931 -> 644 + 653;
-// 0.40M, W = 6, 1024^2: 382 + 458 -> 373 + 415. W = 14 takes about 20 float64 warp instructions a
-// record, 325 cycles of an SM's pipe: 1.2 ms of the 1.65.
+// gridding and degridding in us: 1.03M visibilities, W = 14 cubic, 2048^2: 3194 + 3017 -> 1311 + 1320;
+// 0.81M, W = 7 linear, 2048^2: 726 + 827 -> 349 + 400; 0.40M, W = 9, 256^2: 2450 + 2931 -> 275 + 277;
+// 0.40M, W = 6, 1024^2: 382 + 458 -> 186 + 221. W = 14 takes about 20 float64 warp instructions a
+// record, 325 cycles of an SM's pipe, 1.2 ms in all: the pipe is what bounds it.
 #pragma once
 
 #include "sweep_body.cuh"
