@@ -275,6 +275,16 @@ int grid_from_image(lmg_plan* p, const void* image, void* grid, void* scratch, c
 
 namespace lmg {
 
+std::vector<float> xform_twiddles() {
+  std::vector<float> tw(2 * size_t(kXformN));
+  for (int k = 0; k < kXformN; ++k) {
+    const double a = 2.0 * 3.14159265358979323846 * k / kXformN;
+    tw[2 * size_t(k)] = float(std::cos(a));
+    tw[2 * size_t(k) + 1] = float(std::sin(a));
+  }
+  return tw;
+}
+
 int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t max_vis, int dtype,
                 const PlanOptions& opt, lmg_plan** out) {
   if (!out) return set_error(LMG_EINVAL, "out is NULL");
@@ -386,14 +396,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
     return cuda_error(e, "device query");
   }
   std::vector<float> tw;
-  if (p->xform) {
-    tw.resize(2 * size_t(kXformN));
-    for (int k = 0; k < kXformN; ++k) {
-      const double a = 2.0 * 3.14159265358979323846 * k / kXformN;
-      tw[2 * size_t(k)] = float(std::cos(a));
-      tw[2 * size_t(k) + 1] = float(std::sin(a));
-    }
-  }
+  if (p->xform) tw = xform_twiddles();
   if ((p->xform && (e = cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess) ||
       (e = cudaMemcpy(p->d_table, tab_bytes.data(), tab_bytes.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(p->d_h, h_bytes.data(), h_bytes.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||

@@ -121,5 +121,7 @@ int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64
 void free_plan(lmg_plan* p);
 SweepArgs sweep_args(const lmg_plan* p);
 int cuda_error(cudaError_t e, const char* what);
+// Twiddle table of the fused transforms: (cos, sin) of 2 pi k / kXformN.
+std::vector<float> xform_twiddles();
 
 }  // namespace lmg
