@@ -361,7 +361,7 @@ void free_batch(lmg_batch* b) {
 
 size_t class_smem(const WClass& k, bool degrid, int warps, bool tab_smem) {
   return batch_head_bytes(int(k.chans.size()), k.tab_floats, tab_smem && k.tab_fits) +
-         size_t(warps) * stage_bytes(k.W, 0, degrid);
+         size_t(warps) * stage_bytes(k.W, degrid);
 }
 
 // Shared memory and persistent CTA counts of every W class for the current warps / table

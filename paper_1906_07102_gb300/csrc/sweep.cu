@@ -53,10 +53,9 @@ int ring_slots(int W) { return kD * ((W + kD - 1 + kD - 1) / kD); }
 
 size_t sweep_smem_bytes(int W, int dtype, int Ms, bool table_in_smem, bool degrid, int warps) {
   if (dtype) return warps * sweep64_warp_bytes(W, degrid);
-  const size_t rs = dtype ? 8 : 4;
-  const int Wp = table_stride(W, dtype);
-  const size_t tab = table_in_smem ? align16(size_t(Ms + 1) * Wp * rs) : 0;
-  return tab + size_t(warps) * stage_bytes(W, dtype, degrid);
+  const int Wp = table_stride(W, 0);
+  const size_t tab = table_in_smem ? align16(size_t(Ms + 1) * Wp * sizeof(float)) : 0;
+  return tab + size_t(warps) * stage_bytes(W, degrid);
 }
 
 int sweep_set_smem_limits(int W, int dtype, int accum, size_t smem_bytes, bool degrid, bool ext, bool direct) {
@@ -79,9 +78,8 @@ int sweep_config(int W, int dtype, int Ms, bool degrid, size_t limit, bool* tabl
     *warps = sweep64_warps();
     return 0;
   }
-  const size_t rs = dtype ? 8 : 4;
-  const int Wp = table_stride(W, dtype);
-  *table_in_smem = align16(size_t(Ms + 1) * Wp * rs) <= 96 * 1024;
+  const int Wp = table_stride(W, 0);
+  *table_in_smem = align16(size_t(Ms + 1) * Wp * sizeof(float)) <= 96 * 1024;
   for (int pass = 0; pass < 2; ++pass) {
     for (int w = kWarps; w >= 1; w >>= 1) {
       if (sweep_smem_bytes(W, dtype, Ms, *table_in_smem, degrid, w) <= limit) {
@@ -106,15 +104,9 @@ int grid_launch(const SweepArgs& a, cudaStream_t st) {
   if (!a.direct) {
     // a warp per item, 8 warps per CTA, at most 32 CTAs per SM (items beyond that in turn)
     const int spill_blocks = std::min((a.item_cap + 7) / 8, 32 * kSms);
-    if (a.dtype) {
-      k_grid_spill<double><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
-                                                         static_cast<const double2*>(a.spill),
-                                                         static_cast<double2*>(a.grid), 0);
-    } else {
-      k_grid_spill<float><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
-                                                        static_cast<const float2*>(a.spill),
-                                                        static_cast<float2*>(a.grid), a.accum);
-    }
+    k_grid_spill<float><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
+                                                      static_cast<const float2*>(a.spill),
+                                                      static_cast<float2*>(a.grid), a.accum);
   }
   if (a.accum)
     k_grid_merge<<<2 * kSms, 256, 0, st>>>(a.cuts, a.counters, a.part_cap, a.W, a.N, a.parts,

@@ -4,7 +4,7 @@
 //
 // The grid is cut into strips of S = 32 KC columns; a warp owns one work item (a range of
 // rows of one strip) and lane t owns the KC adjacent columns KC t .. KC t + KC - 1 of the
-// strip (KC = 2 for complex64, 1 for complex128). The item's records come grouped by pairs
+// strip (KC = 2). The item's records come grouped by pairs
 // of support-start rows (dealt inside a pair by the binning, so that 32 consecutive records
 // spread over the pair's columns) and are visited in groups of kD = 2 rows, in chunks of up
 // to 32 records (the records and visibilities of the next two chunks already in flight):
@@ -61,8 +61,8 @@ template <int W> struct Ring {
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
-// Columns per lane: 2 for complex64 (64-column strips), 1 for complex128 (32 columns).
-template <typename R> __host__ __device__ constexpr int cols_per_lane() { return sizeof(R) == 4 ? 2 : 1; }
+// Columns per lane (64-column strips).
+template <typename R> __host__ __device__ constexpr int cols_per_lane() { return 2; }
 
 // Staging layout of one warp.
 template <int W, typename R> struct Lay {
@@ -94,31 +94,22 @@ template <int W, typename R> struct Lay {
   static constexpr size_t degrid_bytes = align16(cv_bytes + align16(u_bytes) + p_bytes);
 };
 
-// Pairs of rows in one register: f32x2 for float (Blackwell's packed FMA), two doubles.
+// Pairs of rows in one register: f32x2 (Blackwell's packed FMA).
 template <typename R> struct PairOf;
 template <> struct PairOf<float> { using T = unsigned long long; };
-template <> struct PairOf<double> { using T = double2; };
 
 __device__ __forceinline__ unsigned long long pfma(unsigned long long a, unsigned long long b, unsigned long long c) {
   return f2fma(a, b, c);
 }
-__device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c) {
-  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
 __device__ __forceinline__ unsigned long long pdup(float x) { return f2pack(x, x); }
-__device__ __forceinline__ double2 pdup(double x) { return make_double2(x, x); }
 template <typename P> __device__ __forceinline__ P pzero();
 template <> __device__ __forceinline__ unsigned long long pzero<unsigned long long>() { return 0ull; }
-template <> __device__ __forceinline__ double2 pzero<double2>() { return make_double2(0.0, 0.0); }
 __device__ __forceinline__ float plo(unsigned long long p) { return f2unpack(p).x; }
 __device__ __forceinline__ float phi(unsigned long long p) { return f2unpack(p).y; }
-__device__ __forceinline__ double plo(double2 p) { return p.x; }
-__device__ __forceinline__ double phi(double2 p) { return p.y; }
 __device__ __forceinline__ float psum(unsigned long long p) {
   const float2 v = f2unpack(p);
   return v.x + v.y;
 }
-__device__ __forceinline__ double psum(double2 p) { return p.x + p.y; }
 
 // Packed error-free addition (Knuth TwoSum on both halves): a receives the rounded sum,
 // lo accumulates the rounding errors (compensated accumulation, complex64 only).
@@ -279,15 +270,10 @@ template <> struct Vec16<float> {
   using T = float4;
   static constexpr int N = 4;
 };
-template <> struct Vec16<double> {
-  using T = double2;
-  static constexpr int N = 2;
-};
 template <typename R> __device__ __forceinline__ R vget(const typename Vec16<R>::T& v, int k);
 template <> __device__ __forceinline__ float vget<float>(const float4& v, int k) {
   return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
 }
-template <> __device__ __forceinline__ double vget<double>(const double2& v, int k) { return k == 0 ? v.x : v.y; }
 
 // The W table weights at one coordinate (row offset `off`, fraction f): nearest / linear
 // rows read with 16-byte loads, or the extended lookups (Lagrange, direct calculation).
@@ -315,14 +301,6 @@ __device__ __forceinline__ void lookup(const R* __restrict__ tab, int Wp, int in
       for (int i = 0; i < W; ++i) c[i] = vget<R>(r0[i / VE], i % VE);
     }
   } else {
-    // direct calculation exists for float64 plans and W <= 11 only (plan creation)
-    if constexpr (sizeof(R) == 8 && W <= 11) {
-      if (interp == 4) {
-#pragma unroll 1
-        for (int i = 0; i < W; ++i) c[i] = direct_entry<R>(tab, W, i, f);
-        return;
-      }
-    }
 #pragma unroll
     for (int i = 0; i < W; ++i) c[i] = lagrange_entry<R>(tab + off + i, Wp, interp, f);
   }
@@ -344,10 +322,7 @@ __device__ __forceinline__ void stage_cv(const R (&cv)[W], int d, R* __restrict_
   V* out = reinterpret_cast<V*>(dst);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    V x;
-    if constexpr (sizeof(R) == 4) x = make_float4(e[4 * v], e[4 * v + 1], e[4 * v + 2], e[4 * v + 3]);
-    else x = make_double2(e[2 * v], e[2 * v + 1]);
-    out[v] = x;
+    out[v] = make_float4(e[4 * v], e[4 * v + 1], e[4 * v + 2], e[4 * v + 3]);
   }
 }
 
@@ -387,13 +362,8 @@ __device__ __forceinline__ void stage_grid(const R* __restrict__ tab, int Wp, in
       v[2 * j + 1] = im;
     }
     unsigned char* dst = rec + ((L0 + m) & (L::PS - 1)) * L::SA;
-    if constexpr (sizeof(R) == 4) {
-      static_assert(KC == 2, "complex64 lanes own two columns");
-      *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < KC; ++j) reinterpret_cast<double2*>(dst)[j] = make_double2(v[2 * j], v[2 * j + 1]);
-    }
+    static_assert(KC == 2, "lanes own two columns");
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
 
@@ -424,8 +394,7 @@ __device__ __forceinline__ void stage_degrid(const R* __restrict__ tab, int Wp, 
       v[j] = c;
     }
     unsigned char* dst = rec + ((L0 + m) & (L::PS - 1)) * L::SU;
-    if constexpr (sizeof(R) == 4 && KC == 2) *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
-    else *reinterpret_cast<R*>(dst) = v[0];
+    *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
   }
 }
 
@@ -493,56 +462,27 @@ template <typename R> struct Fetch {
 
 // Resident CTAs per SM the register allocation must allow.
 template <int W, typename R, bool COMP = false, bool EXT = false> constexpr int min_blocks() {
-  return (sizeof(R) == 4 && W <= 8 && !COMP) ? 2 : 1;
+  return (W <= 8 && !COMP) ? 2 : 1;
 }
 
 // KC complex values of one row of a lane's columns: 16-byte store / load.
 template <typename R, int KC>
 __device__ __forceinline__ void store_cols(typename Cplx<R>::T* dst, const R (&re)[KC], const R (&im)[KC]) {
-  if constexpr (sizeof(R) == 4 && KC == 2) {
-    *reinterpret_cast<float4*>(dst) = make_float4(re[0], im[0], re[1], im[1]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      typename Cplx<R>::T o;
-      o.x = re[j];
-      o.y = im[j];
-      dst[j] = o;
-    }
-  }
+  *reinterpret_cast<float4*>(dst) = make_float4(re[0], im[0], re[1], im[1]);
 }
 // The same added to the grid, one 16-byte reduction where the lane holds anything.
 template <typename R, int KC>
 __device__ __forceinline__ void add_cols(typename Cplx<R>::T* dst, const R (&re)[KC], const R (&im)[KC]) {
-  if constexpr (sizeof(R) == 4 && KC == 2) {
-    if (re[0] != 0.f || im[0] != 0.f || re[1] != 0.f || im[1] != 0.f)
-      red_add2(dst, make_float2(re[0], im[0]), make_float2(re[1], im[1]));
-  } else {
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      typename Cplx<R>::T o;
-      o.x = re[j];
-      o.y = im[j];
-      if (o.x != R(0) || o.y != R(0)) red_add(dst + j, o);
-    }
-  }
+  if (re[0] != 0.f || im[0] != 0.f || re[1] != 0.f || im[1] != 0.f)
+    red_add2(dst, make_float2(re[0], im[0]), make_float2(re[1], im[1]));
 }
 template <typename R, int KC>
 __device__ __forceinline__ void load_cols(const typename Cplx<R>::T* src, R (&re)[KC], R (&im)[KC]) {
-  if constexpr (sizeof(R) == 4 && KC == 2) {
-    const float4 v = *reinterpret_cast<const float4*>(src);
-    re[0] = v.x;
-    im[0] = v.y;
-    re[1] = v.z;
-    im[1] = v.w;
-  } else {
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      const typename Cplx<R>::T v = src[j];
-      re[j] = v.x;
-      im[j] = v.y;
-    }
-  }
+  const float4 v = *reinterpret_cast<const float4*>(src);
+  re[0] = v.x;
+  im[0] = v.y;
+  re[1] = v.z;
+  im[1] = v.w;
 }
 
 // Loads one gridding slot (KC complex a = Cu w V) as (a_re, a_re) and (a_im, a_im) per column,
@@ -550,21 +490,11 @@ __device__ __forceinline__ void load_cols(const typename Cplx<R>::T* src, R (&re
 // the slot loads).
 template <typename R, int KC>
 __device__ __forceinline__ void load_slot(const unsigned char* p, typename PairOf<R>::T (&a)[KC][2]) {
-  if constexpr (sizeof(R) == 4) {
-    static_assert(KC == 2, "complex64 lanes own two columns");
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    a[0][0] = pdup(x.x);
-    a[0][1] = pdup(x.y);
-    a[1][0] = pdup(x.z);
-    a[1][1] = pdup(x.w);
-  } else {
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      const double2 x = reinterpret_cast<const double2*>(p)[j];
-      a[j][0] = pdup(x.x);
-      a[j][1] = pdup(x.y);
-    }
-  }
+  const float4 x = *reinterpret_cast<const float4*>(p);
+  a[0][0] = pdup(x.x);
+  a[0][1] = pdup(x.y);
+  a[1][0] = pdup(x.z);
+  a[1][1] = pdup(x.w);
 }
 
 // Loads the Cv' pairs of record l.
@@ -574,20 +504,14 @@ __device__ __forceinline__ void load_cv_pairs(const unsigned char* s_cv, int l,
   using L = Lay<W, R>;
   constexpr int NPR = Ring<W>::TP / 2;
   const R* p = reinterpret_cast<const R*>(s_cv) + l * L::CVS;
-  if constexpr (sizeof(R) == 4) {
-    const ulonglong2* v = reinterpret_cast<const ulonglong2*>(p);
+  const ulonglong2* v = reinterpret_cast<const ulonglong2*>(p);
 #pragma unroll
-    for (int m = 0; m < NPR / 2; ++m) {
-      const ulonglong2 x = v[m];
-      c[2 * m] = x.x;
-      c[2 * m + 1] = x.y;
-    }
-    if constexpr (NPR % 2) c[NPR - 1] = reinterpret_cast<const unsigned long long*>(p)[NPR - 1];
-  } else {
-    const double2* v = reinterpret_cast<const double2*>(p);
-#pragma unroll
-    for (int m = 0; m < NPR; ++m) c[m] = v[m];
+  for (int m = 0; m < NPR / 2; ++m) {
+    const ulonglong2 x = v[m];
+    c[2 * m] = x.x;
+    c[2 * m + 1] = x.y;
   }
+  if constexpr (NPR % 2) c[NPR - 1] = reinterpret_cast<const unsigned long long*>(p)[NPR - 1];
 }
 
 // One gridding work item (rows [r0, r1) of one strip), run by the 32 lanes of a warp;
@@ -602,7 +526,6 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   using L = Lay<W, R>;
   constexpr int KC = L::KC, S = 32 * KC;
   constexpr int RS = Ring<W>::R, NP = Ring<W>::P, NPR = Ring<W>::TP / 2, RH = RS / 2;
-  static_assert(!COMP || sizeof(R) == 4, "compensated accumulation is for complex64");
   unsigned char* s_cv = my;
   unsigned char* s_a = my + L::cv_bytes;
 
@@ -851,17 +774,7 @@ __device__ __forceinline__ void spill_item(const Item* __restrict__ items, int n
   for (int j = 0; j < kMaxRows; ++j)
     if (j < rows) {
       typename Cplx<R>::T* dst = g + static_cast<size_t>((item.r0 + item.own + j) % N) * N;
-      if constexpr (sizeof(R) == 4 && KC == 2) {
-        red_add2(dst, make_float2(vr[j][0], vi[j][0]), make_float2(vr[j][1], vi[j][1]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < KC; ++c) {
-          typename Cplx<R>::T v;
-          v.x = vr[j][c];
-          v.y = vi[j][c];
-          red_add(dst + c, v);
-        }
-      }
+      red_add2(dst, make_float2(vr[j][0], vi[j][0]), make_float2(vr[j][1], vi[j][1]));
     }
 }
 
@@ -899,13 +812,8 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
   auto put_pair = [&](int h) {
 #pragma unroll
     for (int j = 0; j < KC; ++j) {
-      if constexpr (sizeof(R) == 4) {
-        gR[j][h] = f2pack(nr0[j], nr1[j]);
-        gI[j][h] = f2pack(ni0[j], ni1[j]);
-      } else {
-        gR[j][h] = make_double2(nr0[j], nr1[j]);
-        gI[j][h] = make_double2(ni0[j], ni1[j]);
-      }
+      gR[j][h] = f2pack(nr0[j], nr1[j]);
+      gI[j][h] = f2pack(ni0[j], ni1[j]);
     }
   };
 #pragma unroll
@@ -969,16 +877,11 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
             {
               const unsigned char* p1 = s_u + l1 * L::UP + myslot * L::SU;
               const unsigned char* p2 = s_u + l2 * L::UP + myslot * L::SU;
-              if constexpr (sizeof(R) == 4 && KC == 2) {
-                const float2 x1 = *reinterpret_cast<const float2*>(p1), x2 = *reinterpret_cast<const float2*>(p2);
-                u1[0] = x1.x;
-                u1[1] = x1.y;
-                u2[0] = x2.x;
-                u2[1] = x2.y;
-              } else {
-                u1[0] = *reinterpret_cast<const R*>(p1);
-                u2[0] = *reinterpret_cast<const R*>(p2);
-              }
+              const float2 x1 = *reinterpret_cast<const float2*>(p1), x2 = *reinterpret_cast<const float2*>(p2);
+              u1[0] = x1.x;
+              u1[1] = x1.y;
+              u2[0] = x2.x;
+              u2[1] = x2.y;
             }
             R p1r = R(0), p1i = R(0), p2r = R(0), p2i = R(0);
 #pragma unroll
@@ -1104,28 +1007,27 @@ template <bool EXT> void* sweep_kernel_pick(int W, int accum, bool degrid, bool 
 }
 
 // Staging bytes of one warp (runtime W).
-template <int W> size_t stage_bytes_w(int dtype, bool degrid) {
-  if (dtype) return degrid ? Lay<W, double>::degrid_bytes : Lay<W, double>::grid_bytes;
+template <int W> size_t stage_bytes_w(bool degrid) {
   return degrid ? Lay<W, float>::degrid_bytes : Lay<W, float>::grid_bytes;
 }
-inline size_t stage_bytes(int W, int dtype, bool degrid) {
+inline size_t stage_bytes(int W, bool degrid) {
   switch (W) {
-    case 1: return stage_bytes_w<1>(dtype, degrid);
-    case 2: return stage_bytes_w<2>(dtype, degrid);
-    case 3: return stage_bytes_w<3>(dtype, degrid);
-    case 4: return stage_bytes_w<4>(dtype, degrid);
-    case 5: return stage_bytes_w<5>(dtype, degrid);
-    case 6: return stage_bytes_w<6>(dtype, degrid);
-    case 7: return stage_bytes_w<7>(dtype, degrid);
-    case 8: return stage_bytes_w<8>(dtype, degrid);
-    case 9: return stage_bytes_w<9>(dtype, degrid);
-    case 10: return stage_bytes_w<10>(dtype, degrid);
-    case 11: return stage_bytes_w<11>(dtype, degrid);
-    case 12: return stage_bytes_w<12>(dtype, degrid);
-    case 13: return stage_bytes_w<13>(dtype, degrid);
-    case 14: return stage_bytes_w<14>(dtype, degrid);
-    case 15: return stage_bytes_w<15>(dtype, degrid);
-    case 16: return stage_bytes_w<16>(dtype, degrid);
+    case 1: return stage_bytes_w<1>(degrid);
+    case 2: return stage_bytes_w<2>(degrid);
+    case 3: return stage_bytes_w<3>(degrid);
+    case 4: return stage_bytes_w<4>(degrid);
+    case 5: return stage_bytes_w<5>(degrid);
+    case 6: return stage_bytes_w<6>(degrid);
+    case 7: return stage_bytes_w<7>(degrid);
+    case 8: return stage_bytes_w<8>(degrid);
+    case 9: return stage_bytes_w<9>(degrid);
+    case 10: return stage_bytes_w<10>(degrid);
+    case 11: return stage_bytes_w<11>(degrid);
+    case 12: return stage_bytes_w<12>(degrid);
+    case 13: return stage_bytes_w<13>(degrid);
+    case 14: return stage_bytes_w<14>(degrid);
+    case 15: return stage_bytes_w<15>(degrid);
+    case 16: return stage_bytes_w<16>(degrid);
     default: return 0;
   }
 }
