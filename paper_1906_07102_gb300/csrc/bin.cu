@@ -587,7 +587,10 @@ __global__ void __launch_bounds__(kItemThreads)
   const int pre = base + x - nj;
   // joined pairs go to m items of equal counts, as far as the places to cut allow
   const int m_items = max(1, (joined + target - 1) / target);
-  auto item_of = [&](int r) { return joined ? static_cast<int>(static_cast<long long>(r) * m_items / joined) : 0; };
+  // (pairs after the last record belong to the last item: one of their own would pass the bound)
+  auto item_of = [&](int r) {
+    return joined ? min(m_items - 1, static_cast<int>(static_cast<long long>(r) * m_items / joined)) : 0;
+  };
   s_pre[i] = pre;
   __syncthreads();
   // a joined item starts at the block's first pair, after a cut pair, and where the running
