@@ -238,7 +238,9 @@ __global__ void k_scan_final(const int* __restrict__ in, long long n, const int*
 }
 
 // The whole scan in one CTA, for up to kScanOne buckets (a grid of 1024^2 complex64): at that size
-// each of the two launches above costs more than the work.
+// each of the two launches above costs more than the work, so long as a thread's 16 buckets move as
+// four 16-byte words (binning 20,000 visibilities, 512^2: 26.8 us, 32.9 with the two launches;
+// 1024^2: 30.4 and 34.6, and 38 with single loads here).
 constexpr int kScanOneThreads = 1024;
 constexpr int kScanOne = kScanOneThreads * kScanPer;
 
@@ -246,12 +248,17 @@ __global__ void __launch_bounds__(kScanOneThreads)
     k_scan_one(const int* __restrict__ in, int n, int* __restrict__ offsets) {
   __shared__ int warp_sums[kScanOneThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, base = threadIdx.x * kScanPer;
+  // 16-byte loads and stores: n is a whole number of strips of N >= 64 rows, N a multiple of 32
   int v[kScanPer];
   int s = 0;
 #pragma unroll
-  for (int i = 0; i < kScanPer; ++i) {
-    v[i] = base + i < n ? in[base + i] : 0;
-    s += v[i];
+  for (int i = 0; i < kScanPer; i += 4) {
+    const int4 q = base + i < n ? *reinterpret_cast<const int4*>(in + base + i) : make_int4(0, 0, 0, 0);
+    v[i] = q.x;
+    v[i + 1] = q.y;
+    v[i + 2] = q.z;
+    v[i + 3] = q.w;
+    s += (q.x + q.y) + (q.z + q.w);
   }
   int x = s;
   for (int o = 1; o < 32; o <<= 1) {
@@ -268,9 +275,10 @@ __global__ void __launch_bounds__(kScanOneThreads)
   }
   int run = __shfl_sync(0xffffffffu, t - own, w) + x - s;
 #pragma unroll
-  for (int i = 0; i < kScanPer; ++i) {
-    if (base + i < n) offsets[base + i] = run;
-    run += v[i];
+  for (int i = 0; i < kScanPer; i += 4) {
+    const int4 q = make_int4(run, run + v[i], run + v[i] + v[i + 1], run + v[i] + v[i + 1] + v[i + 2]);
+    if (base + i < n) *reinterpret_cast<int4*>(offsets + base + i) = q;
+    run = q.w + v[i + 3];
   }
   if (threadIdx.x == kScanOneThreads - 1) offsets[n] = run;
 }
@@ -518,6 +526,7 @@ __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale
 // sweep then adds into a zeroed grid; otherwise they store their rows' zeros).
 constexpr int kMaxRowsPerBlock = 512;
 constexpr int kItemThreads = kMaxRowsPerBlock / 2;
+constexpr int kManyBlocks = 4 * kSms;
 constexpr int kDenseUnit = 512;
 // Parts that plain float32 gridding sums in one chain. Its accuracy on dense cells follows the
 // length of its chains; 4.1M visibilities on a 256^2 grid, W = 12, relative image error and time:
@@ -687,7 +696,13 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const int nblk = (a.N + a.rows_per_block - 1) / a.rows_per_block;
   const int ntask = a.n_strips * nblk;
   if (a.rows_per_block > kMaxRowsPerBlock) return -1;
-  const int item_threads = a.rows_per_block <= 256 ? 128 : kItemThreads;
+  // Threads: at least the block's row pairs. With more than kManyBlocks blocks, those of up to 64 rows
+  // take one warp each: wide CTAs and their barriers are then what the launch costs (binning of
+  // 200,000 visibilities: complex128 16384^2, 131,072 blocks, 304 -> 170 us; complex64 2560^2, 1600
+  // blocks, 40 -> 38). With fewer, four warps share the cut pairs of the dense blocks (0.7M on
+  // 256^2, 16 blocks: 66 us, in one warp each 102).
+  const int item_threads =
+      a.rows_per_block <= 64 && ntask > kManyBlocks ? 32 : (a.rows_per_block <= 256 ? 128 : kItemThreads);
   k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty,
                                                a.one_record, a.items,
                                                a.counters, a.item_cap, a.cuts, a.part_cap);

@@ -1,0 +1,60 @@
+"""Where the rules for work items and their routes change (needs a GB300): blocks of rows taken by one
+warp each while items are made. References are the float64 oracle with the same table.
+
+Bars, of the largest cell. Float64 1e-12 (sums of up to 1e5 terms of 53-bit rounding). Float32:
+a term carries at most six roundings of 2^-24 (two interpolated weights, their product with the
+visibility), 3.6e-7, and a plain chain of n terms of one sign drifts by about 2^-25 sqrt(n / 3) of its
+sum, 8e-7 for the 2000 records that chains end with here: 4e-6 for plain sums (four times both),
+1e-6 for compensated ones, whose chains add no more than the last rounding.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import imaging as I  # noqa: E402
+from paper_1906_07102_gb300 import lmg  # noqa: E402
+from paper_1906_07102_gb300 import synthetic as S  # noqa: E402
+from tests.cases import INTERP, caller_table  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"plain": 4e-6, "compensated": 1e-6}
+
+
+def clusters(N, spread, dense, seed):
+    """spread positions over the disk, and dense ones in four pairs of rows of one block around a
+    strip's edge (two next to each other, two apart)."""
+    g = np.random.default_rng(seed)
+    a = S.disk_uniform(spread, 0.45 * N, seed) if spread else np.zeros((0, 2))
+    row = g.choice([4.0, 6.0, 12.0, 20.0], dense)
+    b = np.stack([g.uniform(-1.5, 1.5, dense), row + g.uniform(0.1, 1.9, dense)], 1)
+    uv = np.concatenate([a, b])
+    return np.ascontiguousarray(uv[g.permutation(len(uv))])
+
+
+def check(N, W, interp, dtype, accum, uv, max_vis=None, Ms=200):
+    """Gridding and degridding against the oracle; returns the plan's info."""
+    T = caller_table(W, Ms)
+    p = lmg.Plan(lmg.Table(W, 0.5, Ms, interp, values=T), N // 2, 1.0 / N, max_vis or len(uv), dtype)
+    p.bin(torch.from_numpy(uv).cuda())
+    assert p.status() == (0, 0)
+    vis = 1.0 + 0.3 * S.complex_normal(len(uv), 5)
+    cd, tol = (torch.complex64, TOL[accum]) if dtype == "c64" else (torch.complex128, 1e-12)
+    op = I.Plan(uv[:, 0], uv[:, 1], W, N)
+    ref = I.grid(op, T, Ms, INTERP[interp], vis)
+    g = p.grid(torch.from_numpy(vis).to("cuda", cd), accum=accum).cpu().numpy()
+    assert np.abs(g - ref).max() <= tol * np.abs(ref).max()
+    G = S.random_image(N, 6)
+    d = p.degrid(torch.from_numpy(G).to("cuda", cd)).cpu().numpy()
+    dref = I.degrid(op, T, Ms, INTERP[interp], G)
+    assert np.abs(d - dref).max() <= (1e-5 if dtype == "c64" else 1e-12) * np.abs(dref).max()
+    return p.info()
+
+
+@pytest.mark.parametrize("dtype,accum,N", [
+    ("c64", "plain", 1536), ("c64", "plain", 1600), ("c64", "compensated", 1600),  # 576 and 625 blocks
+    ("c128", "plain", 1088), ("c128", "plain", 1152)])                              # 578 and 648
+def test_blocks_of_rows_in_one_warp(dtype, accum, N):
+    """Above 608 blocks a warp makes a block's items, several cut pairs of rows among them."""
+    check(N, 6, "linear", dtype, accum, clusters(N, 3000, 20000, N))
