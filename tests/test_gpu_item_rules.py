@@ -58,3 +58,10 @@ def check(N, W, interp, dtype, accum, uv, max_vis=None, Ms=200):
 def test_blocks_of_rows_in_one_warp(dtype, accum, N):
     """Above 608 blocks a warp makes a block's items, several cut pairs of rows among them."""
     check(N, 6, "linear", dtype, accum, clusters(N, 3000, 20000, N))
+
+
+@pytest.mark.parametrize("N,spread,dense", [(64, 31, 0), (64, 40, 3000), (512, 4001, 20000), (1152, 3000, 33)])
+@pytest.mark.parametrize("interp", ["nearest", "linear", "cubic"])
+def test_float64_one_cell_supports(N, interp, spread, dense):
+    """W = 1 in float64: a lane a record, several of one warp in one cell, rows with few records."""
+    check(N, 1, interp, "c128", "plain", clusters(N, spread, dense, N + dense))
