@@ -696,13 +696,15 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   const int nblk = (a.N + a.rows_per_block - 1) / a.rows_per_block;
   const int ntask = a.n_strips * nblk;
   if (a.rows_per_block > kMaxRowsPerBlock) return -1;
-  // Threads: at least the block's row pairs. With more than kManyBlocks blocks, those of up to 64 rows
-  // take one warp each: wide CTAs and their barriers are then what the launch costs (binning of
-  // 200,000 visibilities: complex128 16384^2, 131,072 blocks, 304 -> 170 us; complex64 2560^2, 1600
-  // blocks, 40 -> 38). With fewer, four warps share the cut pairs of the dense blocks (0.7M on
-  // 256^2, 16 blocks: 66 us, in one warp each 102).
-  const int item_threads =
-      a.rows_per_block <= 64 && ntask > kManyBlocks ? 32 : (a.rows_per_block <= 256 ? 128 : kItemThreads);
+  // Threads: at least the block's row pairs. On sparse grids with more than kManyBlocks blocks, those of
+  // up to 64 rows take one warp each: wide CTAs and their barriers are then what the launch costs
+  // (binning of 200,000 visibilities: complex128 16384^2, 131,072 blocks, 304 -> 170 us; complex64
+  // 2560^2, 1600 blocks, 40 -> 38). With fewer blocks four warps share the cut pairs of the dense ones
+  // (0.7M on 256^2, 16 blocks: 66 us, in one warp each 102); with dense blocks narrow CTAs, all
+  // resident at once, would place the items in no order (4.1M on 4096^2, gridding and degridding
+  // 529 to 598 us in place of 473 to 534).
+  const bool narrow = a.rows_per_block <= 64 && ntask > kManyBlocks && a.nvis < 256ll * ntask;
+  const int item_threads = narrow ? 32 : (a.rows_per_block <= 256 ? 128 : kItemThreads);
   k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty,
                                                a.one_record, a.items,
                                                a.counters, a.item_cap, a.cuts, a.part_cap);

@@ -56,7 +56,8 @@ def check(N, W, interp, dtype, accum, uv, max_vis=None, Ms=200):
     ("c64", "plain", 1536), ("c64", "plain", 1600), ("c64", "compensated", 1600),  # 576 and 625 blocks
     ("c128", "plain", 1088), ("c128", "plain", 1152)])                              # 578 and 648
 def test_blocks_of_rows_in_one_warp(dtype, accum, N):
-    """Above 608 blocks a warp makes a block's items, several cut pairs of rows among them."""
+    """Above 608 blocks, few visibilities on average: a warp makes a block's items, several cut pairs of
+    rows among them."""
     check(N, 6, "linear", dtype, accum, clusters(N, 3000, 20000, N))
 
 
