@@ -320,10 +320,18 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   p->n_strips = int(N / strip);
   const size_t rs = dtype == LMG_C128 ? 8 : 4;
   p->Wp = table_stride(p->W, dtype);
-  p->direct = dtype == LMG_C128 || (opt.direct && grid_direct(N, dtype));
   p->auto_target = opt.min_item_target == 0;
-  p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block,
-                               p->auto_target ? item_target_for(max_vis, dtype) : opt.min_item_target));
+  const int64_t blocks = item_bound(0, p->n_strips, int(N), opt.min_rows_per_block, 1) - 2;
+  int target = p->auto_target ? item_target_for(max_vis, dtype, p->W, blocks) : opt.min_item_target;
+  // small complex64 grids are added into, but for sparse ones and those whose items are whole blocks
+  // (gridding 60,000 visibilities, W = 9, 2304^2: 39 us stored, 43 added): these want no items below
+  // kMaxItem records, and so no more spill rows than that
+  p->direct = dtype == LMG_C128 || (opt.direct && grid_direct(N));
+  if (dtype == LMG_C64 && p->direct && (grid_sparse(N, max_vis) || (p->W >= kWideSupport && blocks >= kWideWarps))) {
+    p->direct = false;
+    target = kMaxItem;
+  }
+  p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block, target));
   p->part_cap = dtype == LMG_C64 && p->auto_target ? part_bound(max_vis) : 0;
   if (inject_fault("item_cap")) p->item_cap = 1;
   const long long L = (long long)p->n_strips * N;
@@ -478,8 +486,9 @@ int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64
   a.n_strips = p->n_strips;
   a.strip = p->strip;
   a.rows_per_block = p->rows_per_block;
-  a.item_target = p->auto_target ? item_target_within(nvis, p->dtype, p->n_strips, int(p->N), p->rows_per_block, p->item_cap)
+  a.item_target = p->auto_target ? item_target_within(nvis, p->dtype, p->W, p->n_strips, int(p->N), p->rows_per_block, p->item_cap)
                                  : p->item_target;
+  a.part_target = p->auto_target ? part_target_for(nvis, p->dtype, a.item_target) : 4 * a.item_target;
   a.item_cap = p->item_cap;
   a.skip_empty = p->direct ? 1 : 0;
   a.one_record = p->dtype == LMG_C128 ? 1 : 0;

@@ -510,16 +510,17 @@ __global__ void k_bin_scatter_tracks(const double* __restrict__ uv, double scale
 // target below kDenseUnit (few visibilities) they are joined in units of the pairs that W - 1
 // rows take, up to kDenseUnit records: items of whole units meet in a cell at most two at a time,
 // so that their sums do not depend on which is added first. Elsewhere items are cut at any pair,
-// and a pair with 8 target records or more is cut into parts of 4 to 8 target records, one item
+// and a pair with 2 part records or more is cut into parts of one to two times part, one item
 // each: a warp sweeps an item alone, and one dense pair near the uv origin, 40 times the target,
 // is otherwise a serial chain that the whole launch waits for (4.1M visibilities on a 256^2 grid:
 // 512 such items kept a fifth of the resident warps busy, and degridding took 4.4 ms, 0.43 with
 // the cut).
-// fine (complex128): items are cut at any pair, and a pair of 2 target records or more into parts of
-// one to two targets: those sweeps end in tails of long items (see item_target_for), and their sums
+// fine (complex128): items are cut at any pair, and parts are as small as items: those sweeps end in tails of long items (see item_target_for), and their sums
 // meet at the strips' edges in any order anyway.
-// Items per block are at most 1 + count / target: a cut pair of n >= 8 target records gives at
-// most n / (4 target) parts and one more boundary between joined pairs.
+// Items per block are at most 1 + joined / target and, for a cut pair of n >= 2 part records, at most
+// n / part parts and one more boundary between joined pairs: 3 n / (2 part). With part >= 3/2 target
+// (complex64) that is 1 + count / target in all; with part = target (complex128) half as much again,
+// where item_bound allows two records a visibility and there is one.
 // Items with more than target/2 records are placed from the front of the array and the others
 // from the back, so that the sweeps (which take items front to back, then back to front)
 // start the heavy ones first. skip_empty: items without records are left out (the gridding
@@ -551,8 +552,8 @@ __device__ __forceinline__ void put_item(const Item& it, int target, Item* __res
 __device__ __forceinline__ int centre_out(int k, int n) { return n / 2 + ((k & 1) ? -((k + 1) >> 1) : k >> 1); }
 
 __global__ void __launch_bounds__(kItemThreads)
-    k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int skip_empty, int fine,
-                 Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
+    k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int part, int skip_empty,
+                 int fine, Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
   __shared__ int s_off[kItemThreads + 1];  // offset of each pair's first record
   __shared__ int s_pre[kItemThreads];      // records of joined pairs before each pair
   __shared__ unsigned s_start[kItemThreads / 32 + 1], s_cut[kItemThreads / 32];
@@ -576,7 +577,6 @@ __global__ void __launch_bounds__(kItemThreads)
   const int first = in ? unit_first(i) : 0;
   const bool dense = in && dense_unit(first);
   const int n = in ? s_off[i + 1] - s_off[i] : 0;
-  const int part = fine ? target : 4 * target;  // records of a cut pair's part, about
   const bool cut = dense && n >= 2 * part;
   const int nj = cut ? 0 : n;
   int x = nj;
@@ -705,24 +705,43 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   // 529 to 598 us in place of 473 to 534).
   const bool narrow = a.rows_per_block <= 64 && ntask > kManyBlocks && a.nvis < 256ll * ntask;
   const int item_threads = narrow ? 32 : (a.rows_per_block <= 256 ? 128 : kItemThreads);
-  k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.skip_empty,
-                                               a.one_record, a.items,
-                                               a.counters, a.item_cap, a.cuts, a.part_cap);
+  k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.part_target,
+                                               a.skip_empty, a.one_record, a.items, a.counters, a.item_cap, a.cuts,
+                                               a.part_cap);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 // Records per work item. A warp sweeps an item alone, so a call with few visibilities wants
 // small items: with 512 records each, the 20,000 visibilities of a 256^2 grid made 40 items for
-// 2432 resident warps and the sweep took 50 us, as long as one item does. 32 warps per SM give
-// each warp about two items; from 32 records down an item is all start-up (its grid rows and
+// 2432 resident warps and the sweep took 50 us, as long as one item does. 32 items per SM give
+// each warp about two; from 32 records down an item is all start-up (its grid rows and
 // offsets); above 512 nothing is gained (best of {256 .. 2048} on 4.1M-visibility tracks).
+// Between 256 and 512 the second item of some warps becomes a third, and whole 512s are faster: 2.0M
+// visibilities, W = 8, 2048^2, gridding and degridding 123 + 122 us with 411 records, 109 + 108.
+// Supports from kWideSupport on keep half as many warps and read or add W - 1 rows more than an
+// item owns, so that cutting blocks of rows costs more than it balances once there is one for each warp:
+// degridding 200,000 visibilities, W = 12, 4096^2: 149 us with 41 records, 122 with 512; 2.0M: 310 and
+// 260. With fewer blocks it gains (W = 12, 2048^2: 59 us uncut, 50).
 // complex128: 96 items per SM, of which 10 to 32 are swept at a time. A record costs its SM 325
 // cycles at W = 14, an item's rows little beside it: with 32 items per SM, two to three a warp, the
 // float64 pipe stood still for a sixth of the sweep. Gridding and degridding in us: 1.03M visibilities,
 // W = 14 cubic, 2048^2: 1646 + 1666 -> 1311 + 1320; 0.40M, W = 9, 256^2: 644 + 653 -> 275 + 277.
-int item_target_for(long long nvis, int dtype) {
-  const long long t = nvis / ((dtype ? 96 : 32) * kSms);
-  return static_cast<int>(t < 32 ? 32 : (t > 512 ? 512 : t));
+static int per_item(long long nvis, int per_sm) {
+  const long long t = nvis / (per_sm * kSms);
+  return static_cast<int>(t < 32 ? 32 : (t > kMaxItem ? kMaxItem : t));
+}
+
+int item_target_for(long long nvis, int dtype, int W, long long blocks) {
+  if (dtype) return per_item(nvis, 96);
+  const int t = per_item(nvis, 32);
+  if (W >= kWideSupport) return blocks >= kWideWarps ? kMaxItem : t;
+  return t > kMaxItem / 2 ? kMaxItem : t;
+}
+
+int part_target_for(long long nvis, int dtype, int target) {
+  if (dtype) return target;
+  const int t = 4 * per_item(nvis, 32), least = (3 * target + 1) / 2;
+  return t > least ? t : least;
 }
 
 // Work items that nvis positions (two records each at most) can make (see k_make_items).
@@ -738,10 +757,10 @@ int part_bound(long long max_vis) {
   return static_cast<int>((n > max_vis / 512 ? n : max_vis / 512) / 2 + 1);
 }
 
-int item_target_within(long long nvis, int dtype, int n_strips, int N, int rows_per_block, int cap) {
-  const long long room = cap - item_bound(0, n_strips, N, rows_per_block, 1);
+int item_target_within(long long nvis, int dtype, int W, int n_strips, int N, int rows_per_block, int cap) {
+  const long long blocks = item_bound(0, n_strips, N, rows_per_block, 1) - 2, room = cap - blocks - 2;
   const long long least = room > 0 ? (2 * nvis + room - 1) / room : 0;
-  const int t = item_target_for(nvis, dtype);
+  const int t = item_target_for(nvis, dtype, W, blocks);
   return least > t ? static_cast<int>(least) : t;
 }
 

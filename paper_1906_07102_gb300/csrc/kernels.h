@@ -50,7 +50,7 @@ struct BinArgs {
   double scale2;  // N * pixel_scale * 2^32
   int W, N, n_strips, strip;  // strip: columns per strip (strip_width)
   int one_record;  // a support that crosses into the next strip still makes one record (its strip's)
-  int rows_per_block, item_target, item_cap;
+  int rows_per_block, item_target, part_target, item_cap;
   int skip_empty;  // leave out work items without records (gridding into a zeroed grid)
   int max_blocks;
   int* hist;       // n_strips * N, followed by the counters
@@ -81,16 +81,25 @@ int xform_model_launch(const void* image, void* grid, void* scratch, const float
 
 int bin_launch(const BinArgs& a, cudaStream_t st);
 int bin_scan_chunks(long long L);
-int item_target_for(long long nvis, int dtype);
+constexpr int kMaxItem = 512;          // records
+constexpr int kWideSupport = 9;        // from here on the float32 sweeps keep 8 warps per SM, 16 below
+constexpr int kWideWarps = 8 * kSms;   // resident in all
+int item_target_for(long long nvis, int dtype, int W, long long blocks);
+// Records of one part of a cut row pair, about: at least 3/2 target (item_bound).
+int part_target_for(long long nvis, int dtype, int target);
 long long item_bound(long long nvis, int n_strips, int N, int rows_per_block, int target);
 // Parts of cut row pairs that up to max_vis positions can make.
 int part_bound(long long max_vis);
 // item_target_for, raised until item_bound stays within cap items.
-int item_target_within(long long nvis, int dtype, int n_strips, int N, int rows_per_block, int cap);
-// Gridding by adding into a zeroed grid instead of storing whole rows and adding spill rows:
-// complex64 where the grid stays in L2 (129 MB, half of it at most; complex128 always), zeroing and vector reductions cost
-// no DRAM traffic, and small items need no spill buffer and no pass over it.
-constexpr bool grid_direct(long long N, int dtype) { return N * N * (dtype ? 16 : 8) <= (48ll << 20); }
+int item_target_within(long long nvis, int dtype, int W, int n_strips, int N, int rows_per_block, int cap);
+// Gridding by adding into a zeroed grid instead of storing whole rows and adding spill rows, complex64
+// (complex128 always adds): where the grid stays in L2 (129 MB, half of it at most), zeroing and vector
+// reductions cost no DRAM traffic, and small items need no spill buffer and no pass over it.
+constexpr bool grid_direct(long long N) { return N * N * 8 <= (48ll << 20); }
+// Few visibilities for the grid: storing its rows, mostly zeros, as the sweep passes them is then cheaper
+// than zeroing all and adding some. Gridding in us, stored and added: 20,000 on 2496^2 (W = 5) 31 and
+// 38, on 2048^2 33 and 35, on 1600^2 36 and 30; 1000 on 1024^2 (W = 16) 31 and 38.
+constexpr bool grid_sparse(long long N, long long nvis) { return nvis << 18 < N * N * N; }
 
 struct SweepArgs {
   const Rec* recs;

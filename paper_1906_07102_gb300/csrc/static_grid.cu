@@ -32,7 +32,7 @@ constexpr long long kMaxBuckets = static_cast<long long>(kMaxStrips) * kMaxN;
 constexpr int kMaxItems = kMaxStrips * ((kMaxN + kRowsPerBlock - 1) / kRowsPerBlock) +
                           static_cast<int>(2 * kMaxVis / kMinItemTarget) + 2;  // item_bound
 constexpr int kMaxWp = table_stride(16, LMG_C64);  // float row stride for W <= 16
-static_assert(grid_direct(kMaxN, LMG_C64), "every size adds into a zeroed grid: no spill buffer");
+static_assert(grid_direct(kMaxN), "every size adds into a zeroed grid: no spill buffer");
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~size_t(255); }
 
@@ -178,7 +178,8 @@ extern "C" int lmg_grid_static(const lmg_table* t, int64_t n_image, double pixel
   b.n_strips = n_strips;
   b.strip = kStaticStrip;
   b.rows_per_block = kRowsPerBlock;
-  b.item_target = item_target_within(nvis, LMG_C64, n_strips, int(N), kRowsPerBlock, item_cap);
+  b.item_target = item_target_within(nvis, LMG_C64, W, n_strips, int(N), kRowsPerBlock, item_cap);
+  b.part_target = part_target_for(nvis, LMG_C64, b.item_target);
   b.item_cap = item_cap;
   b.skip_empty = 1;
   b.max_blocks = s->sms * 8;

@@ -66,3 +66,24 @@ def test_blocks_of_rows_in_one_warp(dtype, accum, N):
 def test_float64_one_cell_supports(N, interp, spread, dense):
     """W = 1 in float64: a lane a record, several of one warp in one cell, rows with few records."""
     check(N, 1, interp, "c128", "plain", clusters(N, spread, dense, N + dense))
+
+
+@pytest.mark.parametrize("N,W,max_vis,stored", [
+    (512, 7, 511, True), (512, 7, 513, False),              # N^3 / 2^18 = 512
+    (2048, 7, 32767, True), (2048, 7, 32769, False),        # 32768
+    (2176, 9, 200000, False), (2240, 9, 200000, True),      # W >= 9: 1156 and 1225 blocks of rows
+    (2496, 8, 200000, False), (2560, 8, 200000, True)])     # 48 MB
+def test_route_of_gridding(N, W, max_vis, stored):
+    """Rows stored once (every block of rows has an item, empty ones too) or added into a zeroed grid."""
+    info = check(N, W, "linear", "c64", "plain", clusters(N, 0, 30, N), max_vis)
+    assert (info["items"] >= (N // 64) ** 2) == stored
+
+
+@pytest.mark.parametrize("accum", ["plain", "compensated"])
+@pytest.mark.parametrize("N,W,max_vis,stored", [
+    (2496, 8, 0, False), (2560, 8, 0, True), (2560, 3, 0, True), (2240, 16, 0, True), (2048, 16, 0, False),
+    (2560, 8, 200000, True)])  # a plan for more visibilities has smaller items
+def test_cut_pairs_of_both_routes(accum, N, W, max_vis, stored):
+    uv = clusters(N, 2000, 25000, N + W)
+    info = check(N, W, "linear", "c64", accum, uv, max_vis)
+    assert info["items"] >= (N // 64) ** 2 or not stored
