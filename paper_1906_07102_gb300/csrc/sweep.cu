@@ -7,24 +7,25 @@
 namespace lmg {
 namespace {
 
-template <typename R>
-__global__ void k_grid_spill(const Item* __restrict__ items, const int* __restrict__ counters, int item_cap,
-                             int W, int RS, int N, const typename Cplx<R>::T* __restrict__ spill,
-                             typename Cplx<R>::T* __restrict__ grid, int comp) {
-  int nfront;
-  const int total = work_total(counters, item_cap, nfront);
-  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += (gridDim.x * blockDim.x) >> 5)
-    spill_item<R>(items, nfront, item_cap, W, RS, N, 32 * cols_per_lane<R>(), spill, grid, w, threadIdx.x & 31,
-                  comp != 0);
-}
-
-// The parts of cut row pairs, compensated gridding: a warp sums one row of one pair over the
-// pair's parts, their rounding errors apart, and adds the row to the grid once.
-__global__ void k_grid_merge(const Cut* __restrict__ cuts, const int* __restrict__ counters, int part_cap, int W, int N,
-                             const float2* __restrict__ parts, float2* __restrict__ grid) {
+// What gridding leaves to add after the sweep, a warp at a time: the spill rows of the items (none
+// when the sweep added into a zeroed grid), and the parts of cut row pairs, compensated gridding:
+// one row of one pair is summed over the pair's parts, their rounding errors apart, and added to the
+// grid once. One launch for both: a second one costs 3 us, a tenth of gridding 1000 visibilities.
+__global__ void k_grid_spill(const Item* __restrict__ items, const int* __restrict__ counters, int item_cap, int W,
+                            int RS, int N, const float2* __restrict__ spill, float2* __restrict__ grid, int comp,
+                            const Cut* __restrict__ cuts, int part_cap, const float2* __restrict__ parts) {
   constexpr int S = strip_width(0);
-  const int lane = threadIdx.x & 31, total = min(counters[kCntCuts], part_cap) * (W + 1);
-  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += (gridDim.x * blockDim.x) >> 5) {
+  const int lane = threadIdx.x & 31, first = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int warps = (gridDim.x * blockDim.x) >> 5;
+  if (spill != nullptr) {
+    int nfront;
+    const int total = work_total(counters, item_cap, nfront);
+    for (int w = first; w < total; w += warps)
+      spill_item<float>(items, nfront, item_cap, W, RS, N, S, spill, grid, w, lane, comp != 0);
+  }
+  if (comp == 0) return;
+  const int total = min(counters[kCntCuts], part_cap) * (W + 1);
+  for (int w = first; w < total; w += warps) {
     const Cut c = cuts[w / (W + 1)];
     const int row = w % (W + 1);
     const float2* p = parts + (static_cast<size_t>(c.part0) * (W + 1) + row) * (2 * S) + 2 * lane;
@@ -101,16 +102,13 @@ int grid_launch(const SweepArgs& a, cudaStream_t st) {
   SweepArgs args = a;
   void* params[] = {&args};
   if (cudaLaunchKernel(k, dim3(a.grid_blocks), dim3(32 * a.warps), params, smem, st) != cudaSuccess) return -1;
-  if (!a.direct) {
-    // a warp per item, 8 warps per CTA, at most 32 CTAs per SM (items beyond that in turn)
-    const int spill_blocks = std::min((a.item_cap + 7) / 8, 32 * kSms);
-    k_grid_spill<float><<<spill_blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
-                                                      static_cast<const float2*>(a.spill),
-                                                      static_cast<float2*>(a.grid), a.accum);
+  // complex64: a warp per item or cut row, 8 warps per CTA, at most 32 CTAs per SM (the rest in turn)
+  if (!a.direct || a.accum) {
+    const int blocks = a.direct ? 2 * kSms : std::min((a.item_cap + 7) / 8, 32 * kSms);
+    k_grid_spill<<<blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
+                                        a.direct ? nullptr : static_cast<const float2*>(a.spill),
+                                        static_cast<float2*>(a.grid), a.accum, a.cuts, a.part_cap, a.parts);
   }
-  if (a.accum)
-    k_grid_merge<<<2 * kSms, 256, 0, st>>>(a.cuts, a.counters, a.part_cap, a.W, a.N, a.parts,
-                                           static_cast<float2*>(a.grid));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -686,7 +686,7 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   }
   if constexpr (COMP) {
     if (part) {
-      // a part keeps its sums and their rounding errors apart (k_grid_merge): adding the
+      // a part keeps its sums and their rounding errors apart (k_grid_spill): adding the
       // parts' rounded sums in float32 would cost the accuracy that compensation buys. The
       // pair's rows start at zero (stored by its first part).
       if (!DIRECT && item.own != 0) {
