@@ -454,7 +454,11 @@ int launch_sweeps(lmg_batch* b, int op, cudaStream_t s) {
     if (degrid) k_batch_zero<<<dim3(2 * b->sms, n), 256, 0, s>>>(k.d_desc[op]);
     e = cudaLaunchKernel(batch_kernel_for(k.W, degrid), dim3(k.blocks[d]), dim3(32 * b->warps), params, k.smem[d], s);
     if (e != cudaSuccess) return cuda_error(e, "batch: sweep launch");
-    if (!degrid) k_batch_spill<<<dim3(2 * b->sms, n), 256, 0, s>>>(k.d_desc[op]);
+    if (!degrid) {  // a warp per item, 8 warps per CTA
+      int cap = 1;
+      for (int c : k.chans) cap = std::max(cap, b->plans[size_t(c)]->item_cap);
+      k_batch_spill<<<dim3(std::min(2 * b->sms, (cap + 7) / 8), n), 256, 0, s>>>(k.d_desc[op]);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_error(e, "batch: spill / zeroing launch");
   }
   return LMG_OK;
