@@ -23,6 +23,8 @@ thread_local std::string g_error;
 // of the call it stands for, without making that call:
 //   host_alloc    host allocation of a table object           -> LMG_ENOMEM
 //   device_alloc  every device allocation of a plan            -> LMG_ENOMEM
+//   roomy_plan    the buffers of a complex64 plan that are sized for short work items; the plan
+//                 is made with fewer of them (fit_items) instead
 //   cufft_plan    cuFFT plan creation of a plan                -> LMG_ECUFFT
 //   item_cap      plans get a work-item capacity of one item, so that the binning of any
 //                 input with more than one item exceeds it: the binning's own bounds
@@ -86,7 +88,7 @@ namespace lmg {
 void free_plan(lmg_plan* p) {
   if (!p) return;
   void* ptrs[] = {p->d_table, p->d_h, p->hist, p->offsets, p->rank, p->partial, p->recs,
-                  p->items, p->cuts, p->spill, p->parts, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
+                  p->items, p->cuts, p->spill, p->frac, p->work, p->model, p->d_tw, p->xform_tmp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (p->fft_ok) cufftDestroy(p->fft);
@@ -118,7 +120,7 @@ SweepArgs sweep_args(const lmg_plan* p) {
   a.direct = p->direct ? 1 : 0;
   a.part_cap = p->part_cap;
   a.cuts = p->cuts;
-  a.parts = p->parts;
+  a.parts = reinterpret_cast<float2*>(p->rank);
   a.nvis = p->nvis;
   a.frac = p->frac;
   return a;
@@ -285,8 +287,35 @@ std::vector<float> xform_twiddles() {
   return tw;
 }
 
-int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t max_vis, int dtype,
-                const PlanOptions& opt, lmg_plan** out) {
+// Sizes of a plan's items and of the places for merged chains. The places lie in the ranks' memory, which
+// only binning uses. lean: no more than a plan took when items held 512 records throughout.
+static void fit_items(lmg_plan* p, const PlanOptions& opt, bool lean) {
+  const int64_t blocks = item_bound(0, p->n_strips, int(p->N), opt.min_rows_per_block, 1) - 2;
+  int target = p->auto_target ? item_target_for(p->max_vis, p->dtype, p->W, blocks) : opt.min_item_target;
+  // small complex64 grids are added into, but for sparse ones and those whose items are whole blocks
+  // (gridding 60,000 visibilities, W = 9, 2304^2: 39 us stored, 43 added): these want no items below
+  // kMaxItem records, and so no more spill rows than that
+  p->direct = p->dtype == LMG_C128 || (opt.direct && grid_direct(p->N));
+  if (p->dtype == LMG_C64 && p->direct &&
+      (grid_sparse(p->N, p->max_vis) || (p->W >= kWideSupport && blocks >= kWideWarps))) {
+    p->direct = false;
+    target = kMaxItem;
+  }
+  if (lean && !p->direct) target = kMaxItem;
+  p->item_cap = int(item_bound(p->max_vis, p->n_strips, int(p->N), opt.min_rows_per_block, target));
+  p->rank_bytes = size_t(p->max_vis) * sizeof(int2);
+  p->part_cap = 0;
+  if (p->dtype == LMG_C64 && p->auto_target) {
+    const size_t place = size_t(p->W + 1) * 2 * size_t(p->strip) * sizeof(float2);
+    const int most = part_bound(p->max_vis);
+    const size_t want = place * size_t(lean ? 1 : std::min(most, 32 * kSms));
+    if (p->rank_bytes < want) p->rank_bytes = want;
+    p->part_cap = int(std::min<size_t>(p->rank_bytes / place, size_t(most)));
+  }
+}
+
+static int plan_create_sized(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t max_vis, int dtype,
+                             const PlanOptions& opt, bool lean, lmg_plan** out) {
   if (!out) return set_error(LMG_EINVAL, "out is NULL");
   *out = nullptr;
   if (!t) return set_error(LMG_EINVAL, "table is NULL");
@@ -321,18 +350,7 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   const size_t rs = dtype == LMG_C128 ? 8 : 4;
   p->Wp = table_stride(p->W, dtype);
   p->auto_target = opt.min_item_target == 0;
-  const int64_t blocks = item_bound(0, p->n_strips, int(N), opt.min_rows_per_block, 1) - 2;
-  int target = p->auto_target ? item_target_for(max_vis, dtype, p->W, blocks) : opt.min_item_target;
-  // small complex64 grids are added into, but for sparse ones and those whose items are whole blocks
-  // (gridding 60,000 visibilities, W = 9, 2304^2: 39 us stored, 43 added): these want no items below
-  // kMaxItem records, and so no more spill rows than that
-  p->direct = dtype == LMG_C128 || (opt.direct && grid_direct(N));
-  if (dtype == LMG_C64 && p->direct && (grid_sparse(N, max_vis) || (p->W >= kWideSupport && blocks >= kWideWarps))) {
-    p->direct = false;
-    target = kMaxItem;
-  }
-  p->item_cap = int(item_bound(max_vis, p->n_strips, int(N), opt.min_rows_per_block, target));
-  p->part_cap = dtype == LMG_C64 && p->auto_target ? part_bound(max_vis) : 0;
+  fit_items(p, opt, lean);
   if (inject_fault("item_cap")) p->item_cap = 1;
   const long long L = (long long)p->n_strips * N;
   p->nchunks = bin_scan_chunks(L);
@@ -377,14 +395,12 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   if ((rc = dalloc(reinterpret_cast<unsigned char**>(&p->d_table), tab_bytes.size(), "table")) ||
       (rc = dalloc(reinterpret_cast<unsigned char**>(&p->d_h), h_bytes.size(), "correction")) ||
       (rc = dalloc(&p->hist, size_t(L) + kNumCounters, "histogram and counters")) ||
-      (rc = dalloc(&p->offsets, size_t(L) + 1, "offsets")) || (rc = dalloc(&p->rank, size_t(max_vis), "ranks")) ||
+      (rc = dalloc(&p->offsets, size_t(L) + 1, "offsets")) || (rc = dalloc(reinterpret_cast<unsigned char**>(&p->rank), p->rank_bytes, "ranks")) ||
       (rc = dalloc(&p->partial, size_t(p->nchunks), "scan")) || (rc = dalloc(&p->recs, size_t(dtype == LMG_C128 ? max_vis : 2 * max_vis), "records")) ||
       (rc = dalloc(&p->items, size_t(p->item_cap), "items")) ||
       (!p->direct &&
        (rc = dalloc(reinterpret_cast<unsigned char**>(&p->spill), size_t(p->item_cap) * ring_slots(p->W) * strip * c2, "spill"))) ||
-      (p->part_cap > 0 &&
-       ((rc = dalloc(&p->cuts, size_t(p->part_cap), "cut pairs")) ||
-        (rc = dalloc(&p->parts, size_t(p->part_cap) * size_t(p->W + 1) * 2 * size_t(strip), "sums of parts")))) ||
+      (p->part_cap > 0 && (rc = dalloc(&p->cuts, size_t(p->part_cap), "cut pairs"))) ||
       (dtype == LMG_C128 && (rc = dalloc(&p->frac, size_t(max_vis), "quantisation residuals"))) ||
       (opt.work_grid && (rc = dalloc(reinterpret_cast<unsigned char**>(&p->work), size_t(N) * size_t(N) * c2, "work grid"))) ||
       (opt.work_grid && !p->xform &&
@@ -473,6 +489,18 @@ int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t
   }
   *out = p;
   return LMG_OK;
+}
+
+int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t max_vis, int dtype,
+                const PlanOptions& opt, lmg_plan** out) {
+  const bool roomy = !inject_fault("roomy_plan");
+  int rc = roomy ? plan_create_sized(t, n_image, pixel_scale, max_vis, dtype, opt, false, out) : LMG_ENOMEM;
+  // a plan that does not fit with the buffers for short items may fit without
+  if ((rc == LMG_ENOMEM || rc == LMG_ECUFFT) && dtype == LMG_C64 && opt.min_item_target == 0) {
+    clear_error();
+    rc = plan_create_sized(t, n_image, pixel_scale, max_vis, dtype, opt, true, out);
+  }
+  return rc;
 }
 
 int plan_bin(lmg_plan* p, const double* uv, int64_t nvis, cudaStream_t st, int64_t tracks) {

@@ -150,7 +150,7 @@ __global__ void k_batch_spill(const BatchChan* __restrict__ ch) {
   const int lane = threadIdx.x & 31;
   for (int w = gw; w < total; w += (gridDim.x * blockDim.x) >> 5)
     spill_item<float>(a.items, nfront, a.item_cap, a.W, RS, a.N, a.strip, static_cast<const float2*>(a.spill),
-                      static_cast<float2*>(a.grid), w, lane);
+                      static_cast<float2*>(a.grid), w, lane, merged_sums(a.W, false));
 }
 
 // Zeroes every channel's degridding output before the sweep (blockIdx.y = channel): each

@@ -553,7 +553,8 @@ __device__ __forceinline__ int centre_out(int k, int n) { return n / 2 + ((k & 1
 
 __global__ void __launch_bounds__(kItemThreads)
     k_make_items(const int* __restrict__ offsets, int N, int W, int rows_per_block, int target, int part, int skip_empty,
-                 int fine, Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap) {
+                 int fine, Item* __restrict__ items, int* __restrict__ counters, int cap, Cut* __restrict__ cuts, int part_cap,
+                 int per_place) {
   __shared__ int s_off[kItemThreads + 1];  // offset of each pair's first record
   __shared__ int s_pre[kItemThreads];      // records of joined pairs before each pair
   __shared__ unsigned s_start[kItemThreads / 32 + 1], s_cut[kItemThreads / 32];
@@ -619,7 +620,7 @@ __global__ void __launch_bounds__(kItemThreads)
     const int end = m ? 32 * w + __ffs(m) - 1 : np;
     const int cnt = s_off[end] - s_off[i];
     if (cnt > 0 || !skip_empty)
-      put_item(Item{s, rb + 2 * i, rb + 2 * end, cnt, s_off[i], 2 * (end - i), -1, cnt}, target, items, counters, cap);
+      put_item(Item{s, rb + 2 * i, 2 * (end - i), cnt, s_off[i], cnt, cnt, -1}, target, items, counters, cap);
   }
   // cut pairs, a warp each, their parts over its lanes (one after another over the CTA, with a
   // barrier before and after each pair's update of the parts' counter, the 4.1M visibilities of
@@ -630,23 +631,34 @@ __global__ void __launch_bounds__(kItemThreads)
       if (k0++ % nw != warp) continue;
       const int p = 32 * w + __ffs(m) - 1;
       const int o0 = s_off[p], cnt = s_off[p + 1] - o0, parts = cnt / part;
-      int part0 = -1;
-      if (cuts != nullptr) {
+      // merged chains of per_place parts or more, a place each; a single one needs none
+      const int merged = per_place > 0 ? parts / per_place : 0;
+      int place = -1;
+      if (merged > 1) {
         if (lane == 0) {
-          const int q = atomicAdd(counters + kCntParts, parts);
-          part0 = q + parts <= part_cap ? q : -1;
-          if (part0 >= 0) cuts[atomicAdd(counters + kCntCuts, 1)] = Cut{s, rb + 2 * p, q, parts};
+          const int q = atomicAdd(counters + kCntParts, merged);
+          place = q + merged <= part_cap ? q : -1;
+          if (place >= 0) cuts[atomicAdd(counters + kCntCuts, 1)] = Cut{s, rb + 2 * p, q, merged};
           else atomicOr(counters + kCntStatus, kStatusItemOverflow);
         }
-        part0 = __shfl_sync(0xffffffffu, part0, 0);
+        place = __shfl_sync(0xffffffffu, place, 0);
       }
+      // shares of a whole, the first of them one larger: where the k-th begins
+      const int rec = cnt / parts, rec1 = cnt % parts;
+      const int per = merged > 1 ? parts / merged : 1, per1 = merged > 1 ? parts % merged : 0;
+      auto record = [&](int k) { return rec * k + min(k, rec1); };
+      auto first_part = [&](int g) { return per * g + min(g, per1); };
       for (int k = lane; k < parts; k += 32) {
-        const int a = o0 + static_cast<int>(static_cast<long long>(cnt) * k / parts);
-        const int e = o0 + static_cast<int>(static_cast<long long>(cnt) * (k + 1) / parts);
-        const int ce = o0 + static_cast<int>(static_cast<long long>(cnt) * min(k + kChain, parts) / parts);
-        const int chain = k % kChain == 0 ? ce - a : 0;
-        put_item(Item{s, rb + 2 * p, rb + 2 * p + 2, e - a, a, k == 0 ? 2 : 0, part0 < 0 ? -1 : part0 + k, chain}, target,
-                 items, counters, cap);
+        const int a = record(k), e = record(k + 1);
+        const int chain = fine ? e - a : (k % kChain == 0 ? record(min(k + kChain, parts)) - a : 0);
+        int comp = k == 0 ? cnt : 0, part = -1;
+        if (place >= 0) {
+          const int larger = per1 * (per + 1);
+          const int g = k < larger ? k / (per + 1) : per1 + (k - larger) / per;
+          comp = k == first_part(g) ? record(first_part(g + 1)) - a : 0;
+          part = place + g;
+        }
+        put_item(Item{s, rb + 2 * p, k == 0 ? 2 : 0, e - a, o0 + a, chain, comp, part}, target, items, counters, cap);
       }
     }
   }
@@ -705,9 +717,10 @@ int bin_launch(const BinArgs& a, cudaStream_t st) {
   // 529 to 598 us in place of 473 to 534).
   const bool narrow = a.rows_per_block <= 64 && ntask > kManyBlocks && a.nvis < 256ll * ntask;
   const int item_threads = narrow ? 32 : (a.rows_per_block <= 256 ? 128 : kItemThreads);
+  const int per_place = a.part_cap > 0 ? (part_bound(a.nvis) + a.part_cap - 1) / a.part_cap : 0;
   k_make_items<<<ntask, item_threads, 0, st>>>(a.offsets, a.N, a.W, a.rows_per_block, a.item_target, a.part_target,
                                                a.skip_empty, a.one_record, a.items, a.counters, a.item_cap, a.cuts,
-                                               a.part_cap);
+                                               a.part_cap, per_place);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -28,18 +28,21 @@ __host__ __device__ __forceinline__ int rec_pack(int row, int xrel) { return (ro
 __host__ __device__ __forceinline__ int rec_xrel(int rx) { return static_cast<int>(static_cast<signed char>(rx & 0xff)); }
 __host__ __device__ __forceinline__ int rec_row(int rx) { return static_cast<int>(static_cast<unsigned>(rx) >> 8); }
 
-// Work item: the records [rb, rb + nrec) of rows [r0, r1) of one strip. A pair of rows with
-// many records is cut into several items over the same rows (parts); own (the rows whose final
-// sums the item stores itself, r1 - r0 or 0) is non-zero for the first of them only. part is
-// the part's place in the buffer that compensated sums of parts are kept in, -1 otherwise.
-// Plain float32 gridding takes kChain parts of a pair as one chain: chain is the chain's records
-// for its first part, 0 for the others (which it skips), and nrec for the other items.
+// Work item: the records [rb, rb + nrec) of some rows of one strip from r0 on. A pair of rows with
+// many records is cut into several items over the same rows (parts); own is the number of rows whose
+// final sums the item stores itself: all of its rows, or 0 for a pair's later parts.
+// Gridding takes several parts of a pair as one chain. chain: records of the chain that starts here,
+// plain sums (kChain parts); comp: the same for merged sums (Cut); 0 where an earlier part's chain
+// holds the item's records, nrec for items that are no parts. part: place of a merged chain's sums, -1
+// where it has none (the pair is one chain, added like any item).
 struct alignas(16) Item {
-  int strip, r0, r1, nrec;
-  int rb, own, part, chain;
+  int strip, r0, own, nrec;
+  int rb, chain, comp, part;
+  __device__ __forceinline__ int rows() const { return own ? own : 2; }
 };
 
-// A cut pair of rows r0, r0 + 1: its parts' places are [part0, part0 + parts).
+// A pair of rows r0, r0 + 1 whose chains' sums are merged (compensated gridding): they lie
+// at places part0 to part0 + parts - 1.
 struct alignas(16) Cut {
   int strip, r0, part0, parts;
 };

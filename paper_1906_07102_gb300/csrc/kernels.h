@@ -55,11 +55,11 @@ struct BinArgs {
   int max_blocks;
   int* hist;       // n_strips * N, followed by the counters
   int* offsets;    // n_strips * N + 1
-  int2* rank;      // max_vis: rank of the record(s) in their buckets
+  int2* rank;      // max_vis: rank of the record(s) in their buckets (gridding reuses the memory: SweepArgs::parts)
   int* partial;    // scan chunk sums
   Rec* recs;       // 2 * max_vis
   Item* items;     // item_cap
-  Cut* cuts;       // part_cap or NULL (no compensated gridding): the cut row pairs
+  Cut* cuts;       // part_cap or NULL (no merged chains): the cut row pairs
   int part_cap;
   int* counters;   // kNumCounters, at hist + n_strips * N
   double2* frac;   // max_vis or NULL: per visibility (u_q - u, v_q - v) in cells, the residual
@@ -122,9 +122,9 @@ struct SweepArgs {
   const void* weights;
   void* grid;
   void* spill;        // item_cap * ring rows * strip complex (not used when direct)
-  int part_cap;
-  const Cut* cuts;    // compensated gridding: cut row pairs and the sums of their parts,
-  float2* parts;      // [part][W + 1 rows][sum, rounding error][strip]
+  int part_cap;       // merged chains there can be, 0 for none
+  const Cut* cuts;    // their row pairs and their sums, [place][W + 1 rows][sum, rounding error][strip]
+  float2* parts;
   // degridding
   const void* grid_in;
   void* vis_out;

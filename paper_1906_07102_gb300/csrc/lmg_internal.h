@@ -81,10 +81,10 @@ struct lmg_plan {
   int* partial = nullptr;
   lmg::Rec* recs = nullptr;
   lmg::Item* items = nullptr;
-  // compensated gridding: cut row pairs and the sums of their parts
+  // merged chains of cut row pairs: the pairs, and how many chains' sums fit into the ranks' memory
+  size_t rank_bytes = 0;
   int part_cap = 0;
   lmg::Cut* cuts = nullptr;
-  float2* parts = nullptr;
   int* counters = nullptr;
   void* spill = nullptr;
   double2* frac = nullptr;   // float64 plans: quantisation residual of every position

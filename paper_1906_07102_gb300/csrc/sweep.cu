@@ -8,11 +8,10 @@ namespace lmg {
 namespace {
 
 // What gridding leaves to add after the sweep, a warp at a time: the spill rows of the items (none
-// when the sweep added into a zeroed grid), and the parts of cut row pairs, compensated gridding:
-// one row of one pair is summed over the pair's parts, their rounding errors apart, and added to the
-// grid once. One launch for both: a second one costs 3 us, a tenth of gridding 1000 visibilities.
+// when the sweep added into a zeroed grid), and the merged chains of cut row pairs: one row of one pair
+// is summed over the pair's chains, their rounding errors apart, and added to the grid once. One launch for both: a second one costs 3 us, a tenth of gridding 1000 visibilities.
 __global__ void k_grid_spill(const Item* __restrict__ items, const int* __restrict__ counters, int item_cap, int W,
-                            int RS, int N, const float2* __restrict__ spill, float2* __restrict__ grid, int comp,
+                            int RS, int N, const float2* __restrict__ spill, float2* __restrict__ grid, int merged,
                             const Cut* __restrict__ cuts, int part_cap, const float2* __restrict__ parts) {
   constexpr int S = strip_width(0);
   const int lane = threadIdx.x & 31, first = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -21,9 +20,8 @@ __global__ void k_grid_spill(const Item* __restrict__ items, const int* __restri
     int nfront;
     const int total = work_total(counters, item_cap, nfront);
     for (int w = first; w < total; w += warps)
-      spill_item<float>(items, nfront, item_cap, W, RS, N, S, spill, grid, w, lane, comp != 0);
+      spill_item<float>(items, nfront, item_cap, W, RS, N, S, spill, grid, w, lane, merged != 0);
   }
-  if (comp == 0) return;
   const int total = min(counters[kCntCuts], part_cap) * (W + 1);
   for (int w = first; w < total; w += warps) {
     const Cut c = cuts[w / (W + 1)];
@@ -103,11 +101,13 @@ int grid_launch(const SweepArgs& a, cudaStream_t st) {
   void* params[] = {&args};
   if (cudaLaunchKernel(k, dim3(a.grid_blocks), dim3(32 * a.warps), params, smem, st) != cudaSuccess) return -1;
   // complex64: a warp per item or cut row, 8 warps per CTA, at most 32 CTAs per SM (the rest in turn)
-  if (!a.direct || a.accum) {
+  const bool merged = merged_sums(a.W, a.accum != 0) && a.part_cap > 0;
+  if (!a.direct || merged) {
     const int blocks = a.direct ? 2 * kSms : std::min((a.item_cap + 7) / 8, 32 * kSms);
     k_grid_spill<<<blocks, 256, 0, st>>>(a.items, a.counters, a.item_cap, a.W, ring_slots(a.W), a.N,
                                         a.direct ? nullptr : static_cast<const float2*>(a.spill),
-                                        static_cast<float2*>(a.grid), a.accum, a.cuts, a.part_cap, a.parts);
+                                        static_cast<float2*>(a.grid), merged_sums(a.W, a.accum != 0) ? 1 : 0, a.cuts,
+                                         merged ? a.part_cap : 0, a.parts);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -452,10 +452,13 @@ __global__ void __launch_bounds__(kThreads64) k_sweep64(const SweepArgs a) {
   const int total = work_total(a.counters, a.item_cap, nfront);
   for (int w = next_item(work, lane); w < total; w = next_item(work, lane)) {
     const Item item = a.items[item_slot(w, nfront, a.item_cap)];
-    if constexpr (W == 1 && DEGRID) degrid_item64_cells<EXT>(a, my, item, lane);
-    else if constexpr (W == 1) grid_item64_cells<EXT>(a, my, item, lane);
-    else if constexpr (DEGRID) degrid_item64<W, EXT>(a, my, item, lane);
-    else grid_item64<W, EXT>(a, my, item, lane);
+    if constexpr (DEGRID) {
+      if constexpr (W == 1) degrid_item64_cells<EXT>(a, my, item, lane);
+      else degrid_item64<W, EXT>(a, my, item, lane);
+    } else {
+      if constexpr (W == 1) grid_item64_cells<EXT>(a, my, item, lane);
+      else grid_item64<W, EXT>(a, my, item, lane);
+    }
   }
 }
 

@@ -407,7 +407,7 @@ __device__ __forceinline__ void zero_bytes(unsigned char* p, int bytes, int lane
 // end offset of pair 32 b + t (the offset of row min(r0 + 2 (32 b + t + 1), r1), or the end of
 // the item's records when it holds a part of a pair).
 __device__ __forceinline__ int pair_ends(const int* __restrict__ off, const Item& item, int rend, int b, int lane) {
-  return min(off[min(item.r0 + 2 * (32 * b + lane + 1), item.r1)], rend);
+  return min(off[item.r0 + min(2 * (32 * b + lane + 1), item.rows())], rend);
 }
 
 // Lanes L0 .. L1 (inclusive) intersected with [0, 32).
@@ -514,7 +514,11 @@ __device__ __forceinline__ void load_cv_pairs(const unsigned char* s_cv, int l,
   if constexpr (NPR % 2) c[NPR - 1] = reinterpret_cast<const unsigned long long*>(p)[NPR - 1];
 }
 
-// One gridding work item (rows [r0, r1) of one strip), run by the 32 lanes of a warp;
+// Gridding whose chains of a cut pair are merged in their order instead of added to the grid one by one:
+// compensated sums, for their accuracy.
+__host__ __device__ constexpr bool merged_sums(int W, bool comp) { return comp; }
+
+// One gridding work item (rows of one strip), run by the 32 lanes of a warp;
 // `my` is the warp's staging area in shared memory, `tab` the table (shared or global).
 // DIRECT: the rows are added to a zeroed grid instead of stored, with no spill rows (compiled
 // apart: with both ends in one kernel the 4.1M-visibility sweep took 241 us instead of 224).
@@ -549,13 +553,20 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   const Item item = a.items[slot];
   const int* __restrict__ off = a.offsets + static_cast<long long>(item.strip) * N;
   const int col0 = item.strip * S + KC * lane;
-  const int nrows = item.r1 - item.r0;
-  if (!COMP && item.chain == 0 && item.nrec > 0) return;  // in the chain of an earlier part
-  const bool part = COMP && item.part >= 0;
-  // where the item's rows go: the grid, or for a later chain of a cut pair its spill rows
-  C2* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
-  const bool own = DIRECT || item.own != 0;
-  C2* rows = own ? grid + static_cast<size_t>(item.r0) * N + col0 : sp;
+  constexpr bool MERGED = merged_sums(W, COMP);
+  const int len = MERGED ? item.comp : item.chain;
+  const bool skip = len == 0 && item.nrec > 0;  // in the chain of an earlier part
+  if constexpr (!COMP) {
+    if (skip) return;
+  }
+  // (compensated sums pass over it without rows: a return here costs the W = 16 kernel its registers)
+  const int nrows = COMP && skip ? 0 : item.rows();
+  const bool part = MERGED && !skip && item.part >= 0;
+  // where the item's rows go: the grid, or for a later chain of a cut pair its spill rows (a merged
+  // one's sums go to its place)
+  const bool own = DIRECT || MERGED || item.own != 0;
+  C2* rows = own ? grid + static_cast<size_t>(item.r0) * N + col0
+                 : spill + static_cast<size_t>(slot) * RS * S + KC * lane;
   const int row_stride = own ? N : S;
   // ring pair h holds relative rows 2h' and 2h' + 1 (h' = h mod RH) of the lane's columns
   P accR[KC][RH], accI[KC][RH];
@@ -588,7 +599,7 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   // software pipeline over 32-record windows of the item (window k = records
   // rb + 32k .. rb + 32k + 31, lane l holding record rb + 32k + l): while window k is
   // processed, the visibilities of window k+1 and the records of window k+2 are in flight
-  const int rb = item.rb, rend = item.rb + (COMP ? item.nrec : item.chain);
+  const int rb = item.rb, rend = item.rb + len;
   int pend = pair_ends(off, item, rend, 0, lane);
   int wbase = rb, cstart = rb;
   int last = -(1 << 20);  // the last group that held records: rows up to last + W + 1 hold sums
@@ -684,10 +695,10 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
       }
     }
   }
-  if constexpr (COMP) {
+  if constexpr (MERGED) {
     if (part) {
-      // a part keeps its sums and their rounding errors apart (k_grid_spill): adding the
-      // parts' rounded sums in float32 would cost the accuracy that compensation buys. The
+      // a merged chain keeps its sums and their rounding errors apart (k_grid_spill): adding the
+      // chains' rounded sums in float32 would cost the accuracy that compensation buys. The
       // pair's rows start at zero (stored by its first part).
       if (!DIRECT && item.own != 0) {
         const R zero[KC] = {};
@@ -705,8 +716,11 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
             for (int j = 0; j < KC; ++j) {
               sr[j] = d ? phi(accR[j][h]) : plo(accR[j][h]);
               si[j] = d ? phi(accI[j][h]) : plo(accI[j][h]);
-              er[j] = d ? phi(loR[j][h]) : plo(loR[j][h]);
-              ei[j] = d ? phi(loI[j][h]) : plo(loI[j][h]);
+              er[j] = ei[j] = R(0);
+              if constexpr (COMP) {
+                er[j] = d ? phi(loR[j][h]) : plo(loR[j][h]);
+                ei[j] = d ? phi(loI[j][h]) : plo(loI[j][h]);
+              }
             }
             store_cols<R, KC>(p + (2 * h + d) * (2 * S), sr, si);
             store_cols<R, KC>(p + (2 * h + d) * (2 * S) + S, er, ei);
@@ -728,7 +742,7 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
         if (past < W - 1 && nrows + past <= last + W) {
           R orr[KC], oi[KC];
           ring_row(h, d, orr, oi);
-          add_cols<R, KC>(grid + static_cast<size_t>((item.r1 + past) % N) * N + col0, orr, oi);
+          add_cols<R, KC>(grid + static_cast<size_t>((item.r0 + nrows + past) % N) * N + col0, orr, oi);
         }
       }
     }
@@ -736,9 +750,10 @@ __device__ __forceinline__ void grid_item(const SweepArgs& a, const R* __restric
   }
   // spill: ring pair h holds relative rows nrows + ((2h - nrows) mod RS) (and the next);
   // the W - 1 rows after the item carry partial sums
+  C2* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
 #pragma unroll
   for (int h = 0; h < RH; ++h) {
-    if (h == 0 && item.own == 0) continue;
+    if (h == 0 && !own) continue;
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       R orr[KC], oi[KC];
@@ -757,13 +772,13 @@ template <typename R>
 __device__ __forceinline__ void spill_item(const Item* __restrict__ items, int nfront, int item_cap, int W, int RS,
                                            int N, int S, const typename Cplx<R>::T* __restrict__ spill,
                                            typename Cplx<R>::T* __restrict__ grid, int w, int lane,
-                                           bool comp = false) {  // comp: every part has its own sums
+                                           bool merged) {  // merged_sums of the sweep
   constexpr int kMaxRows = 17;  // 2 + W - 1 for W <= 16
   constexpr int KC = cols_per_lane<R>();
   const int slot = item_slot(w, nfront, item_cap);
   const Item item = items[slot];
-  if ((comp ? item.nrec : item.chain) == 0 || (comp && item.part >= 0)) return;
-  const int rows = item.r1 - item.r0 - item.own + W - 1;
+  if ((merged ? item.comp : item.chain) == 0 || (merged && item.part >= 0)) return;
+  const int rows = item.rows() - item.own + W - 1;
   const typename Cplx<R>::T* sp = spill + static_cast<size_t>(slot) * RS * S + KC * lane;
   R vr[kMaxRows][KC], vi[kMaxRows][KC];
 #pragma unroll
@@ -799,7 +814,7 @@ __device__ __forceinline__ void degrid_item(const SweepArgs& a, const R* __restr
   if (item.nrec == 0) return;
   const int* __restrict__ off = a.offsets + static_cast<long long>(item.strip) * N;
   const int col0 = item.strip * S + KC * lane;
-  const int nrows = item.r1 - item.r0;
+  const int nrows = item.rows();
   // ring pair h holds grid rows item.r0 + 2h' and + 1 (h' = h mod RH) of the lane's columns;
   // rows 0 .. TP - 3 are loaded up front; each group moves the pair that completes its
   // window into the ring (loaded during the previous group) and loads the next group's

@@ -87,3 +87,29 @@ def test_cut_pairs_of_both_routes(accum, N, W, max_vis, stored):
     uv = clusters(N, 2000, 25000, N + W)
     info = check(N, W, "linear", "c64", accum, uv, max_vis)
     assert info["items"] >= (N // 64) ** 2 or not stored
+
+
+def test_memory_of_a_plan_for_many_visibilities():
+    """Records (two of 16 bytes a visibility) and ranks (8 bytes); items, bucket counts and the transforms
+    of a 256^2 grid take a few MB. Sums of cut pairs' chains need nothing of their own at this count."""
+    nvis = 16 << 20
+    tab = lmg.Table(12, 0.5, 200, "linear", values=caller_table(12, 200))
+    lmg.Plan(tab, 128, 1.0 / 256, 1000, "c64")  # the library's own first allocations
+    used = []
+    for _ in range(5):  # other processes' allocations show in the device's free memory too
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        p = lmg.Plan(tab, 128, 1.0 / 256, nvis, "c64")
+        used.append(before - torch.cuda.mem_get_info()[0])
+        assert p.info()["N"] == 256
+        del p
+    assert 0 < min(u for u in used if u > 0) <= 40 * nvis + (32 << 20)
+
+
+@pytest.mark.parametrize("accum", ["plain", "compensated"])
+@pytest.mark.parametrize("N,W", [(64, 16), (64, 3), (256, 8), (2560, 7), (2560, 2)])
+def test_plan_without_room_for_short_items(monkeypatch, accum, N, W):
+    """The sizes a plan falls back to when memory is short: few places for merged chains, several parts of a
+    dense pair in each, and on the stored route no spill rows for items below 512 records."""
+    monkeypatch.setenv("LMG_INJECT_FAULT", "roomy_plan")
+    check(N, W, "linear", "c64", accum, clusters(N, 3000, 40000, N + W), 1 << 17)
