@@ -305,7 +305,8 @@ static void fit_items(lmg_plan* p, const PlanOptions& opt, bool lean) {
   p->item_cap = int(item_bound(p->max_vis, p->n_strips, int(p->N), opt.min_rows_per_block, target));
   p->rank_bytes = size_t(p->max_vis) * sizeof(int2);
   p->part_cap = 0;
-  if (p->dtype == LMG_C64 && p->auto_target) {
+  // W <= 3: no merged chains, and no launch to merge them, below 2^15 visibilities (a pair is then one chain)
+  if (p->dtype == LMG_C64 && p->auto_target && !(p->W <= 3 && p->max_vis < 32768)) {
     const size_t place = size_t(p->W + 1) * 2 * size_t(p->strip) * sizeof(float2);
     const int most = part_bound(p->max_vis);
     const size_t want = place * size_t(lean ? 1 : std::min(most, 32 * kSms));

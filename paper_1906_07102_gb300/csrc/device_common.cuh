@@ -41,7 +41,7 @@ struct alignas(16) Item {
   __device__ __forceinline__ int rows() const { return own ? own : 2; }
 };
 
-// A pair of rows r0, r0 + 1 whose chains' sums are merged (compensated gridding): they lie
+// A pair of rows r0, r0 + 1 whose chains' sums are merged (compensated gridding, and W <= 3): they lie
 // at places part0 to part0 + parts - 1.
 struct alignas(16) Cut {
   int strip, r0, part0, parts;

@@ -515,8 +515,9 @@ __device__ __forceinline__ void load_cv_pairs(const unsigned char* s_cv, int l,
 }
 
 // Gridding whose chains of a cut pair are merged in their order instead of added to the grid one by one:
-// compensated sums, for their accuracy.
-__host__ __device__ constexpr bool merged_sums(int W, bool comp) { return comp; }
+// compensated sums for their accuracy, and supports of up to three rows, whose items, pairs of rows at
+// least, then still meet in a cell two at a time, so that the sums do not depend on the run.
+__host__ __device__ constexpr bool merged_sums(int W, bool comp) { return comp || W <= 3; }
 
 // One gridding work item (rows of one strip), run by the 32 lanes of a warp;
 // `my` is the warp's staging area in shared memory, `tab` the table (shared or global).

@@ -113,3 +113,19 @@ def test_plan_without_room_for_short_items(monkeypatch, accum, N, W):
     dense pair in each, and on the stored route no spill rows for items below 512 records."""
     monkeypatch.setenv("LMG_INJECT_FAULT", "roomy_plan")
     check(N, W, "linear", "c64", accum, clusters(N, 3000, 40000, N + W), 1 << 17)
+
+
+@pytest.mark.parametrize("W", [1, 2, 3])
+@pytest.mark.parametrize("accum", ["plain", "compensated"])
+@pytest.mark.parametrize("N,nvis", [(64, 20000), (64, 300000), (2560, 100000)])
+def test_dense_pairs_of_narrow_supports_sum_in_one_order(W, accum, N, nvis):
+    """Items are pairs of rows at least, so that with W <= 3 two of them meet in a cell: the same bits on
+    every call, however many parts a pair is swept in."""
+    tab = lmg.Table(W, 0.5, 200, "linear", values=caller_table(W, 200))
+    p = lmg.Plan(tab, N // 2, 1.0 / N, nvis, "c64")
+    p.bin(torch.from_numpy(clusters(N, nvis // 2, nvis // 2, W)).cuda())
+    vis = torch.from_numpy(S.complex_normal(nvis, 3)).to("cuda", torch.complex64)
+    first = torch.view_as_real(p.grid(vis, accum=accum))
+    assert p.status() == (0, 0)
+    for _ in range(6):
+        assert torch.equal(first, torch.view_as_real(p.grid(vis, accum=accum)))
