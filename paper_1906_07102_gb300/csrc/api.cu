@@ -494,10 +494,10 @@ static int plan_create_sized(const lmg_table* t, int64_t n_image, double pixel_s
 
 int plan_create(const lmg_table* t, int64_t n_image, double pixel_scale, int64_t max_vis, int dtype,
                 const PlanOptions& opt, lmg_plan** out) {
-  const bool roomy = !inject_fault("roomy_plan");
-  int rc = roomy ? plan_create_sized(t, n_image, pixel_scale, max_vis, dtype, opt, false, out) : LMG_ENOMEM;
+  const bool lean = dtype == LMG_C64 && opt.min_item_target == 0;  // can be made with less
+  int rc = !(lean && inject_fault("roomy_plan")) ? plan_create_sized(t, n_image, pixel_scale, max_vis, dtype, opt, false, out) : LMG_ENOMEM;
   // a plan that does not fit with the buffers for short items may fit without
-  if ((rc == LMG_ENOMEM || rc == LMG_ECUFFT) && dtype == LMG_C64 && opt.min_item_target == 0) {
+  if ((rc == LMG_ENOMEM || rc == LMG_ECUFFT) && lean) {
     clear_error();
     rc = plan_create_sized(t, n_image, pixel_scale, max_vis, dtype, opt, true, out);
   }
