@@ -188,10 +188,12 @@ int lmg_plan_dropped(lmg_plan* p, int64_t* dropped, void* stream);
  *   accum    LMG_ACCUM_PLAIN, or LMG_ACCUM_COMPENSATED (C64 only: each accumulator is
  *            a float pair updated with an error-free sum)
  *   grid     device complex [N][N]; every cell is overwritten (no pre-zeroing needed)
- * Allocates nothing. Where work items are shorter than W - 1 rows (dense rows), the partial
- * rows of two items are added into the same cells by atomics in either order, and so are the
- * cells around a strip's edge for LMG_C128: two calls on the same input may differ at the
- * rounding level of the dtype. */
+ * Allocates nothing. Two calls on the same binning may differ at the rounding level of the
+ * dtype where more than two partial sums are added into a cell by atomics, in any order:
+ * LMG_C64, supports of W >= 4, where the records that W - 1 rows of a strip start exceed
+ * about 512 (or the plan's items are cut at any row, from 1.2 million visibilities on, and
+ * then where items are shorter than W - 1 rows), and in dense pairs of rows, swept in several
+ * parts; LMG_C128, wherever several items meet, at their ends and around the strips' edges. */
 int lmg_grid(lmg_plan* p, const void* vis, const void* weights, int accum, void* grid,
              void* stream);
 
@@ -330,9 +332,9 @@ void* lmg_work_grid(lmg_plan* p);
  * a real-time pipeline that must not allocate while it runs. The paper has no
  * counterpart; this is a deployment variant of the existing path.
  *
- * All working memory (bucket ranks, records, bucket counts, work items,
- * spill rows and the float32 copy of the table) lives in one fixed-size __device__ array
- * of this library, about 16 MB, which every GPU that loads the library holds until the
+ * All working memory (bucket ranks, records, bucket counts, work items and the float32
+ * copy of the table) lives in one fixed-size __device__ array of this library, about
+ * 12 MB, which every GPU that loads the library holds until the
  * process exits.
  * Limits: nvis <= LMG_STATIC_MAX_VIS, grid N = n_image / x0 a multiple of 64 in
  * [64, LMG_STATIC_MAX_N], table oversample <= LMG_STATIC_MAX_OVERSAMPLE; larger sizes

@@ -140,9 +140,5 @@ __device__ __forceinline__ void red_add2(float2* p, float2 a, float2 b) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y)
                : "memory");
 }
-__device__ __forceinline__ void red_add(double2* p, double2 v) {
-  atomicAdd(&p->x, v.x);
-  atomicAdd(&p->y, v.y);
-}
 
 }  // namespace lmg

@@ -9,8 +9,8 @@ namespace lmg {
 // Nodes k = 0..Ng of the direct calculation's folded sums (Ng = 32, Appendix A).
 constexpr int kDirectNodes = 33;
 
-// Strip width of the binning and the sweeps: one lane per two columns for complex64 (64),
-// one lane per column for complex128 (32). dtype 0 = complex64, 1 = complex128.
+// Strip width of the binning and the sweeps: 64 columns for complex64 (two a lane), 32 for
+// complex128 (rows in shared memory). dtype 0 = complex64, 1 = complex128.
 __host__ __device__ constexpr int strip_width(int dtype) { return dtype ? 32 : 64; }
 
 // Row stride (reals) of a device table: rows start on 16-byte boundaries and take an odd
@@ -113,7 +113,7 @@ struct SweepArgs {
   int dtype;          // 0 float, 1 double
   int accum;          // 0 plain, 1 compensated (float only)
   int item_cap;
-  int direct;         // gridding adds into a zeroed grid (grid_direct); else rows are stored once
+  int direct;         // gridding adds into a zeroed grid; else rows are stored once
   int grid_blocks;    // persistent CTAs
   int warps;          // warps per CTA (1..8)
   int table_in_smem;

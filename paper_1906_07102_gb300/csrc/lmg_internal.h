@@ -64,7 +64,7 @@ struct lmg_plan {
   // item_target_for(nvis) (up to 512: best of {64..512} rows x {256..2048} records on the
   // 4.1M-visibility tracks) when auto_target
   bool auto_target = true;
-  bool direct = false;  // gridding adds into a zeroed grid (grid_direct); no spill buffer
+  bool direct = false;  // gridding adds into a zeroed grid (fit_items); no spill buffer
   int n_strips = 0, strip = 64, rows_per_block = 64, item_target = 512, item_cap = 0, nchunks = 0;
   int64_t max_vis = 0, nvis = -1;
   int device = 0, sms = 0;

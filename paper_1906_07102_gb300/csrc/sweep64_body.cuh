@@ -88,7 +88,7 @@ __device__ __forceinline__ double weight64(const double* __restrict__ tab, int W
                                            const double* __restrict__ b) {
   if constexpr (EXT) {
     if constexpr (W <= 11) {
-      if (interp == 4) return direct_entry<double>(tab, W, e, b[0]);
+      if (interp == 4) return direct_entry(tab, W, e, b[0]);
     }
     const double* p = tab + off + e;
     const double c = b[0] * p[0] + b[32] * p[Wp] + b[64] * p[2 * Wp];

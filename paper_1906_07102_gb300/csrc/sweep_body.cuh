@@ -25,15 +25,17 @@
 //      (Cv'_q, Cv'_q+1) x (a, a) with one packed FMA per pair and per real/imaginary part --
 //      the ring index is compile-time, the group loop being unrolled over one ring period.
 //      After a group its kD rows are final and stored as whole rows (512-byte coalesced
-//      stores for complex64). The W-1 rows past the item go to a spill buffer and are added
-//      by k_grid_spill once all items have stored their rows.
+//      stores), the W-1 rows past the item going to a spill buffer that k_grid_spill adds
+//      once all items have stored their rows; or, DIRECT, both are added to a zeroed grid
+//      (fit_items in api.cu says which). Parts of a dense pair: see Item and merged_sums;
 //      degridding: the ring holds grid rows of the lane's columns; the lane forms
 //      sum_q Cv'_q G[row0 + q][c] for its columns, weights them by its Cu slot and stages the
 //      sum in the record's partial-sum slot; the record's lane adds its slots and adds the
 //      result to the zeroed output (a visibility whose support crosses a strip has two
 //      records, one per strip).
-// Every grid cell is written exactly once by the gridding sweep (no pre-zeroing, no
-// shared-memory atomics); only the spill rows are added with global vector atomics.
+// Where rows are stored, every grid cell is written exactly once by the sweep (no pre-zeroing);
+// spill rows, and all rows of a DIRECT sweep, are added with global vector reductions. No
+// shared-memory atomics.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -171,10 +173,6 @@ __device__ __forceinline__ void table_coord(int Wp, int Ms, int interp, unsigned
       off = static_cast<int>((Pm + 0x80000000ull) >> 32) * Wp;
       f = R(0);
     }
-  } else if (interp == 4) {
-    // direct calculation: the coefficients replace the rows; f = s
-    off = 0;
-    f = static_cast<R>(S) * static_cast<R>(2.3283064365386962890625e-10);
   } else {
     // degree d = interp: first stencil row k0 = floor(t - (d - 1) / 2), clamped to
     // [0, Ms - d], and f = t - k0 in [0, d] (t = S Ms 2^-32)
@@ -217,35 +215,31 @@ __device__ __forceinline__ void table_coord_exact(int Wp, int Ms, int interp, un
   }
 }
 
-// Row offsets and fractions of a record for both axes (exact coordinates for float64 plans
-// that carry quantisation residuals).
+// Row offsets and fractions of a record for both axes (exact coordinates for float64 plans, which
+// carry quantisation residuals).
 template <typename R, bool EXT>
 __device__ __forceinline__ void record_coords(const SweepArgs& a, const Rec& rc, int& ou, R& fu, int& ov, R& fv) {
   if constexpr (sizeof(R) == 8) {
-    if (a.frac != nullptr) {
-      const double2 dl = a.frac[rc.idx];
-      table_coord_exact<EXT>(a.Wp, a.Ms, a.interp, rc.su, dl.x, ou, fu);
-      table_coord_exact<EXT>(a.Wp, a.Ms, a.interp, rc.sv, dl.y, ov, fv);
-      return;
-    }
+    const double2 dl = a.frac[rc.idx];
+    table_coord_exact<EXT>(a.Wp, a.Ms, a.interp, rc.su, dl.x, ou, fu);
+    table_coord_exact<EXT>(a.Wp, a.Ms, a.interp, rc.sv, dl.y, ov, fv);
+  } else {
+    table_coord<R, EXT>(a.Wp, a.Ms, a.interp, rc.su, ou, fu);
+    table_coord<R, EXT>(a.Wp, a.Ms, a.interp, rc.sv, ov, fv);
   }
-  table_coord<R, EXT>(a.Wp, a.Ms, a.interp, rc.su, ou, fu);
-  table_coord<R, EXT>(a.Wp, a.Ms, a.interp, rc.sv, ov, fv);
 }
 
 // Direct calculation (Section 5.2, float64 plans): C_a(s) = sum_k alpha[a][k] cos(k phi s) +
 // beta[a][k] sin(k phi s), coef = {phi, alpha[W][33], beta[W][33]} (A^-1 and the node sums
 // folded in on the host); cos/sin(k phi s) by rotation from one sincos.
-template <typename R>
-__device__ __forceinline__ R direct_entry(const R* __restrict__ coef, int W, int a, R s) {
-  R sn, cs;
-  if constexpr (sizeof(R) == 8) sincos(coef[0] * s, &sn, &cs);
-  else sincosf(coef[0] * s, &sn, &cs);
-  const R* al = coef + 1 + a * kDirectNodes;
-  const R* be = coef + 1 + (W + a) * kDirectNodes;
-  R ck = R(1), sk = R(0), acc = al[0];
+__device__ __forceinline__ double direct_entry(const double* __restrict__ coef, int W, int a, double s) {
+  double sn, cs;
+  sincos(coef[0] * s, &sn, &cs);
+  const double* al = coef + 1 + a * kDirectNodes;
+  const double* be = coef + 1 + (W + a) * kDirectNodes;
+  double ck = 1.0, sk = 0.0, acc = al[0];
   for (int k = 1; k < kDirectNodes; ++k) {
-    const R c2 = ck * cs - sk * sn;
+    const double c2 = ck * cs - sk * sn;
     sk = ck * sn + sk * cs;
     ck = c2;
     acc += al[k] * ck + be[k] * sk;
