@@ -144,7 +144,9 @@ int lmg_correction_export(const lmg_table* t, int64_t n_image, int single_precis
  *   max_vis      capacity: the largest nvis later passed to lmg_plan_bin (>= 1)
  *   dtype        LMG_C64 or LMG_C128
  * Allocates the device table, correction factors, binning buffers sized for max_vis, a
- * work grid [N][N] and a cuFFT plan; uses the current CUDA device. Synchronous.
+ * work grid [N][N] and a cuFFT plan; uses the current CUDA device. Synchronous. A plan
+ * whose buffers for short work items do not fit is made without them (larger items: the
+ * same results to rounding, gridding and degridding slower for few visibilities).
  * Returns LMG_EINVAL, LMG_ENOMEM, LMG_ECUDA or LMG_ECUFFT on failure. */
 int lmg_plan_create(const lmg_table* t, int64_t n_image, double pixel_scale,
                     int64_t max_vis, int dtype, lmg_plan** out);
